@@ -936,6 +936,8 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
 
   tc_fence_before();
   __syncthreads();
+  // (the merge waits for this grid's end all the same; let go at the kernel's start, its waiting blocks slowed this kernel)
+  release_dependents();
   if (warp == 0) tmem_dealloc(tb, DecCfg::kTmemCols);
 }
 

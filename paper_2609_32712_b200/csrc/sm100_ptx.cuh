@@ -6,6 +6,7 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace mala {
@@ -108,6 +109,25 @@ template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("set
 
 // generic-proxy writes to shared memory made visible to the async proxy (TMA, tcgen05.mma)
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// ------------------------------------------------------------------------------------------------
+// programmatic dependent launch: a kernel lets its dependents be launched before it has finished; a dependent waits until
+// the kernels before it have finished and their writes are visible (both are no-ops in a plain launch)
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launches `kernel`, which begins with wait_for_primary(), as a programmatic dependent of the kernel before it.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = stream;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // ------------------------------------------------------------------------------------------------
 // TMA tiled loads (no multicast), completion on an mbarrier
