@@ -202,7 +202,9 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   __shared__ int t_page[NG][8][8];                              // small pages: the up to eight pages of tile g
   // the scales of the tile in S^T slot g & 3 (S warp -> softmax); small pages: one per page, and the largest V scale
   __shared__ float sc_k[NG][4][8], sc_v[NG][4][8], sc_vmax[NG][4];
-  __shared__ float q_inv[NG][2][8];        // 2^-k of the query rows of a stream's item
+  // 2^-k of the query rows of a stream's item (item number & 7): the S warp runs up to four tiles, which may be four
+  // items of one tile, ahead of the softmax group, which takes an item's values only after handing its first scores back
+  __shared__ float q_inv[NG][8][8];
   __shared__ __align__(16) float xch[NG][2][2][4][16];     // [stream][half][buffer][warp][row maxima 0..7, row sums 8..15]
   __shared__ __align__(16) float st_m[NG][2][8], st_l[NG][2][8], st_y[NG][2][8];   // a finished item's (m, l, yref)
   __shared__ int st_r[NG][2];                              // ... and its retained tiles
@@ -422,7 +424,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           const int r2 = HALF + qh;
           *reinterpret_cast<uint32_t*>(q8 + qh * 128 + (((e0 >> 4) ^ (qh & 7)) << 4) + (e0 & 15)) = s01.x | (s23.x << 16);
           *reinterpret_cast<uint32_t*>(q8 + r2 * 128 + (((e0 >> 4) ^ (r2 & 7)) << 4) + (e0 & 15)) = s01.y | (s23.y << 16);
-          if (lane == 0) q_inv[k][ip][qh] = down;
+          if (lane == 0) q_inv[k][ne & 7][qh] = down;
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -747,7 +749,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         if (lane == 0) mbar_arrive(&s_free[k][sb]);
         if (t == 0) {
 #pragma unroll
-          for (int q = 0; q < GS; ++q) c2q[q] = c2 * *(volatile float*)&q_inv[k][ip][hb + q];
+          for (int q = 0; q < GS; ++q) c2q[q] = c2 * *(volatile float*)&q_inv[k][ne & 7][hb + q];
         }
         const int kpos = (j0 - t) * 128 + kt;
         float x[GS], tmax[GS];

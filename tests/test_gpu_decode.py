@@ -359,6 +359,17 @@ def test_decode_fp8_cache_many_work_items_per_cta(mala, oracle, B, Nk, S, Hq, Hk
 
 
 @pytest.mark.parametrize("tau", [0.0, 1e-4])
+@pytest.mark.parametrize("B,Nk,S", [(300, 256, 2), (40, 2048, 16)])
+def test_decode_fp8_one_tile_items_with_queries_of_different_magnitudes(mala, oracle, B, Nk, S, tau):
+    # work items of one tile: the scores of several items ahead are formed while the group still works on an earlier one,
+    # each with its own power-of-two scale of the query rows
+    w = W.custom_decode(B, 4, 2, Nk, 64, S, seed=B)
+    f = 2.0 ** torch.randint(-3, 2, (B, 1, 4, 1), generator=torch.Generator().manual_seed(B)).float()
+    w["q"] = (w["q"].float() * f).to(torch.bfloat16)
+    _run_fp8(mala, oracle, w, tau, S, rounding_bound=True)
+
+
+@pytest.mark.parametrize("tau", [0.0, 1e-4])
 def test_decode_fp8_repeated_launches_give_identical_bits(mala, tau):
     """Several work items per CTA, eight tiles each, launched many times: the result does not depend on how the groups
     of a CTA happen to interleave (no atomics on the data path, every hand-over through a barrier)."""
