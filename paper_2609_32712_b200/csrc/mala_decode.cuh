@@ -173,6 +173,8 @@ inline int decode_launch_with_scratch(mala_tin q, mala_tin kc, mala_tin vc, mala
   p.Sq = Sq;
   p.B = B; p.Hq = Hq; p.Hkv = Hkv; p.Nk = Nk; p.tps = tps; p.num_splits = num_splits; p.words = (tps + 31) / 32;
   p.n_items = B * Hkv * num_splits;
+  p.by_splits.set((uint32_t)num_splits);
+  p.by_hkv.set((uint32_t)Hkv);
   p.scale_log2 = scale * 1.4426950408889634f;
   p.log2_tau = tau > 0.f ? log2f(tau) : -INFINITY;
   if (p.bitmask &&
@@ -184,6 +186,7 @@ inline int decode_launch_with_scratch(mala_tin q, mala_tin kc, mala_tin vc, mala
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return MALA_ERR_CUDA;
   const int grid = p.n_items < sms ? p.n_items : sms;   // persistent: one CTA per SM
+  p.sched = decode_sched_fits(B, p.n_items, grid, 1, D == 256 ? DecCfgT<256>::kSchedItems : DecCfg::kSchedItems);
   const int R = G * Sq;   // rows of a work item
 #define MALA_DEC_LAUNCH3(DENSE, GP, MULTI)                                                                           \
   {                                                                                                                  \
@@ -269,6 +272,7 @@ inline int decode_fp8_launch(mala_tin q, mala_tin kc, mala_tin vc, const float* 
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return MALA_ERR_CUDA;
   const int grid = p.n_items < sms ? p.n_items : sms;
+  p.sched = decode_sched_fits(B, p.n_items, grid, 2, DecF8Cfg<2, false>::kSchedItems);   // (two streams)
 #define MALA_F8_LAUNCH(DENSE, GP)                                                                                      \
   do {                                                                                                                  \
     if (Sq > 1) mala_decode_fp8_kernel<DENSE, GP, false, 2, false, true><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p); \

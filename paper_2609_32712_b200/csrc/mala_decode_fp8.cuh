@@ -55,25 +55,6 @@
 
 namespace mala {
 
-// Division of a 32-bit number by a divisor known at launch, as a multiplication and shifts (every role works out for
-// itself which sequence, KV head and split a work item is; hardware has no integer divide, and the few dozen
-// dependent instructions of an emulated one would sit on the per-tile chain of the softmax threads).
-struct FastDiv {
-  uint32_t d, mul, sh;
-  __host__ void set(uint32_t divisor) {
-    d = divisor;
-    uint32_t l = 0;
-    while ((1ull << l) < divisor) ++l;
-    sh = l;
-    mul = (uint32_t)(((1ull << 32) * ((1ull << l) - divisor)) / divisor + 1);
-  }
-  __device__ __forceinline__ uint32_t div(uint32_t n) const {
-    if (d == 1u) return n;
-    const uint32_t t = __umulhi(mul, n);
-    return (t + ((n - t) >> 1)) >> (sh - 1u);
-  }
-};
-
 struct DecF8Params {
   float* o_part;                 // [B, Hq, num_splits, 128] fp32, normalised per split
   float* lse_part;               // [B, Hq, num_splits] natural log; -inf for an empty split
@@ -86,6 +67,7 @@ struct DecF8Params {
   int B, Hq, Hkv, Nk, tps, num_splits, words, n_items, nt;
   float scale_log2, log2_tau;
   FastDiv by_splits, by_hkv;
+  int sched;                     // items in the order of decode_schedule
   // paged cache (block_table != null): K / V are [num_pages, page_size, Hkv, d], the scales [num_pages, Hkv, tpp];
   // Nk = max_pages * page_size lays out the splits, a sequence holds seqlens[b] keys (null: Nk)
   const int32_t* block_table;    // [B, max_pages]
@@ -121,6 +103,7 @@ struct DecF8Cfg {
   static constexpr int kSmemBytes = kGroups * kStreamBytes + 1024;
   static constexpr int kHalves = kSplit_ ? 2 : 1;        // warpgroups of a stream's softmax group
   static constexpr int kThreads = 32 * (4 * kGroups) + 128 * kGroups * kHalves + 128;   // issuing warps, softmax groups, epilogue group
+  static constexpr int kSchedItems = 256;                // entries of a CTA's list of items
   static constexpr uint32_t kColsPerStream = 96;         // S^T ring 4 x 16, O^T 2 x 16 (item parity)
   static constexpr uint32_t kTmemCols = kGroups * kColsPerStream <= 128 ? 128 : 256;
 };
@@ -208,6 +191,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   __shared__ __align__(16) float xch[NG][2][2][4][16];     // [stream][half][buffer][warp][row maxima 0..7, row sums 8..15]
   __shared__ __align__(16) float st_m[NG][2][8], st_l[NG][2][8], st_y[NG][2][8];   // a finished item's (m, l, yref)
   __shared__ int st_r[NG][2];                              // ... and its retained tiles
+  __shared__ uint16_t sched[Cfg::kSchedItems];   // the CTA's items when p.sched
   __shared__ int early_exit;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -227,6 +211,9 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   for (int k = 0; k < NG; ++k)   // Q8 and P8^T rows that are never written stay zero
     for (int i = tid; i < (2 * Cfg::kQ8Bytes + PP * Cfg::kP8Bytes) / 16; i += Cfg::kThreads)
       reinterpret_cast<uint4*>(sQ8_of(k))[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (p.sched)   // (its tables lie in the K ring, which nothing has been copied into yet)
+    decode_schedule<NG, Cfg::kThreads>(sched, reinterpret_cast<int*>(sKr_of(0)), kPaged ? p.seqlens : nullptr, p.B, p.Hkv,
+                                       p.num_splits, p.tps, p.Nk, p.n_items);
   fence_proxy_async_smem();
   if (tid == 0) {
     early_exit = (*(volatile int*)status != 0);
@@ -294,13 +281,16 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     split = bs - b * p.num_splits;
     j0 = split * p.tps + T - 1;
   };
-  // the CTA's work items are blockIdx.x, + gridDim.x, ..; stream k takes the k-th, (k + NG)-th, .. of them
-  const int item_step = NG * (int)gridDim.x;
+  // the CTA's y-th work item (>= n_items: none); stream k takes y = k, k + NG, ..
+  const int n_mine = (p.n_items + NG * (int)gridDim.x - 1) / (NG * (int)gridDim.x) * NG;
+  auto item_at = [&](int y) -> int {
+    if (p.sched) return y < n_mine ? (int)sched[y] : p.n_items;
+    return (int)blockIdx.x + y * (int)gridDim.x;
+  };
 
   if (warp < 4 * NG) {
     // ------------------------------------------------------------------ the issuing warps of stream k
     const int job = warp / NG, k = warp - job * NG;
-    const int item0 = (int)blockIdx.x + k * (int)gridDim.x;
     uint8_t* sKr = sKr_of(k);
     uint8_t* sVr = sVr_of(k);
     uint8_t* sQ8 = sQ8_of(k);
@@ -315,7 +305,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       //      warp-uniform); lane c looks up the page of copy c and issues that copy
       if (lane == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); }
       int ne = 0, g = 0;
-      for (int item = item0; item < p.n_items && ok; item += item_step) {
+      for (int y = k, item; ok && (item = item_at(y)) < p.n_items; y += NG) {
         const int T = tiles_of(item);
         if (T == 0) continue;
         int b, hkv, split, j0;
@@ -354,7 +344,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       if (lane == 0) {
         tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
         int ne = 0, g = 0;
-        for (int item = item0; item < p.n_items && ok; item += item_step) {
+        for (int y = k, item; ok && (item = item_at(y)) < p.n_items; y += NG) {
           const int T = tiles_of(item);
           if (T == 0) continue;
           int b, hkv, split, j0;
@@ -393,7 +383,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       const uint64_t dQ0 = make_smem_desc(smem_u32(sQ8), 16, 1024);
       const uint64_t dK0 = make_smem_desc(smem_u32(sKr), 16, 1024);
       int ne = 0, g = 0;
-      for (int item = item0; item < p.n_items && ok; item += item_step) {
+      for (int y = k, item; ok && (item = item_at(y)) < p.n_items; y += NG) {
         const int T = tiles_of(item);
         if (T == 0) continue;
         const int ip = ne & 1;
@@ -482,7 +472,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       // ---- the votes (MALA kernel): a retained tile's raw V copy is requested, the decision is passed on
       if (!kDense) {
         int g = 0, nv = 0;                       // tiles so far; raw V copies requested -- ring slot nv % NV
-        for (int item = item0; item < p.n_items && ok; item += item_step) {
+        for (int y = k, item; ok && (item = item_at(y)) < p.n_items; y += NG) {
           const int T = tiles_of(item);
           if (T == 0) continue;
           int b, hkv, split, j0;
@@ -527,7 +517,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       // P8^T read MN-major too, without swizzle: 16 bytes (the 16 columns) per key, core matrices of 8 keys 128 bytes apart
       const uint64_t dP0 = make_smem_desc(smem_u32(sP), 128, 128) & ~((uint64_t)7 << 61);
       int ne = 0, g = 0, npv = 0;                // items, tiles, PVs so far: raw V stage npv % NV, P8^T slot npv % PP
-      for (int item = item0; item < p.n_items && ok; item += item_step) {
+      for (int y = k, item; ok && (item = item_at(y)) < p.n_items; y += NG) {
         const int T = tiles_of(item);
         if (T == 0) continue;
         const int ip = ne & 1;
@@ -583,7 +573,9 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     for (int i = 0; i < NG; ++i) ne_k[i] = 0;
     bool ok = true;
     int k = 0;
-    for (int item = (int)blockIdx.x; item < p.n_items && ok; item += (int)gridDim.x, k = (k + 1 == NG) ? 0 : k + 1) {
+    for (int y = 0; y < n_mine && ok; ++y, k = (k + 1 == NG) ? 0 : k + 1) {
+      const int item = item_at(y);
+      if (item >= p.n_items) continue;           // (one stream may have an item less than the other)
       const int T = tiles_of(item);
       int b, hkv, split, j0;
       geometry(item, b, hkv, split, j0, T);
@@ -645,7 +637,6 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     const int k = (warp - 4 * NG) / (4 * HS);
     const int half = kSplit ? (((warp - 4 * NG) >> 2) & 1) : 0;   // which four of the (up to) eight heads
     const int hb = half * 4;
-    const int item0 = (int)blockIdx.x + k * (int)gridDim.x;
     uint8_t* sP = sP_of(k);
     const uint32_t colS = (uint32_t)k * Cfg::kColsPerStream, colO0 = colS + 64u;
     const int w = warp & 3;
@@ -692,7 +683,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       }
       return true;
     };
-    for (int item = item0; item < p.n_items && ok; item += item_step) {
+    for (int y = k, item; ok && (item = item_at(y)) < p.n_items; y += NG) {
       const int T = tiles_of(item);
       if (T == 0) continue;
       int b, hkv, split, j0;

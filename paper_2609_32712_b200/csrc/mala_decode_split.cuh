@@ -28,6 +28,7 @@
 // the V tile's coordinates to the UMMA warp) and every sequence may have its own length (which then takes the
 // place of Nk in the item geometry, in L and in the mask of the newest tile).
 #pragma once
+#include "mala_decode_sched.cuh"
 #include "sm100_ptx.cuh"
 
 namespace mala {
@@ -48,6 +49,8 @@ struct DecParams {
                                  // per page
   int Sq;                        // new tokens per sequence (the last Sq positions of the cache); rows = Sq * Hq/Hkv
   int B, Hq, Hkv, Nk, tps, num_splits, words, n_items;   // Nk: longest cache the splits are laid out for
+  int sched;                     // items in the order of decode_schedule
+  FastDiv by_splits, by_hkv;
   float scale_log2, log2_tau;
 };
 
@@ -62,6 +65,7 @@ struct DecCfgT {
   static constexpr int kKStages = D > 128 ? 2 : 3, kVStages = D > 128 ? 1 : 3, kPStages = 4, kSStages = 4;
   static constexpr int kSmemBytes = 2 * kQBytes + (kKStages + kVStages) * kTileBytes + kPStages * kPBytes + 1024;
   static constexpr int kThreads = 384;                   // producer, UMMA warp, two idle warps, up to two softmax groups
+  static constexpr int kSchedItems = D > 128 ? 128 : 512; // entries of a CTA's list of items (256 columns leave 368 bytes)
   static constexpr uint32_t kTmemCols = 128;             // S^T ring 4 x 16, O^T 2 x 16 (item parity), O^T of channels 128.. 2 x 16
   static constexpr uint32_t kColO = 64, kColOHi = 96;
 };
@@ -148,6 +152,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   __shared__ int v_row[8], v_outer[8];     // TMA coordinates of the V tile of tile g (ring; written by the producer;
                                            // pages smaller than a tile: sequence and key block instead)
   __shared__ __align__(16) float xch_max[2][2][4][8], xch_sum[2][2][4][8];   // [buffer][group][warp][row]: per-tile exchange
+  __shared__ uint16_t sched[DecCfg::kSchedItems];   // the CTA's items when p.sched
   __shared__ int early_exit;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -159,6 +164,8 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   for (int i = tid; i < 2 * DecCfg::kQBytes / 16; i += DecCfg::kThreads) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0u, 0u, 0u, 0u);
   // likewise the rows R..15 of the P^T ring, so that those columns of O^T stay finite
   for (int i = tid; i < DecCfg::kPStages * DecCfg::kPBytes / 16; i += DecCfg::kThreads) reinterpret_cast<uint4*>(sP)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (p.sched)   // (its tables lie in the K ring, which nothing has been copied into yet)
+    decode_schedule<1, DecCfg::kThreads>(sched, reinterpret_cast<int*>(sK), p.seqlens, p.B, p.Hkv, p.num_splits, p.tps, p.Nk, p.n_items);
   fence_proxy_async_smem();
   if (tid == 0) {
     early_exit = (*(volatile int*)status != 0);
@@ -185,13 +192,22 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   tc_fence_after();
   const uint32_t tb = tmem_base_s;
 
-  // geometry of work item `item`: batch, KV head, split, number of legal tiles, newest key block, keys of the
-  // sequence
+  // the CTA's y-th work item (>= n_items: no more)
+  const int n_mine = (p.n_items + (int)gridDim.x - 1) / (int)gridDim.x;
+  auto item_at = [&](int y) -> int {
+    if (p.sched) return y < n_mine ? (int)sched[y] : p.n_items;
+    return (int)blockIdx.x + y * (int)gridDim.x;
+  };
+  // geometry of work item `item`: batch, KV head, split, number of legal tiles, newest key block, keys of the sequence.
+  // The KV head is the fastest index of an item's number: CTAs side by side then read the same rows of a key-major cache.
+  // It is rotated by one from split to split, so that a CTA's items are spread over the heads (which may retain very
+  // different shares of their tiles) also where the number of CTAs and the number of heads have common factors.
   auto geometry = [&](int item, int& b, int& hkv, int& split, int& T, int& j0, int& nk) {
-    split = item % p.num_splits;
-    const int bh = item / p.num_splits;
-    hkv = bh % p.Hkv;
-    b = bh / p.Hkv;
+    const int bs = (int)p.by_hkv.div((uint32_t)item);
+    hkv = item - bs * p.Hkv + bs;
+    hkv -= (int)p.by_hkv.div((uint32_t)hkv) * p.Hkv;
+    b = (int)p.by_splits.div((uint32_t)bs);
+    split = bs - b * p.num_splits;
     nk = p.seqlens ? min(p.Nk, max(0, __ldg(p.seqlens + b))) : p.Nk;
     const int lo = split * p.tps * 128;
     const int hi = min(nk, lo + p.tps * 128);
@@ -237,7 +253,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     int ne = 0, g = 0, ks = 0, vs = 0;
     uint32_t kpar = 1, vpar = 1;
     bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+    for (int y = 0, item; ok && (item = item_at(y)) < p.n_items; ++y) {
       int b, hkv, split, T, j0, nk;
       geometry(item, b, hkv, split, T, j0, nk);
       if (T == 0) continue;
@@ -281,7 +297,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
       int ks = 0, vs = 0;
       uint32_t kpar = 1, vpar = 1;              // "empty" parities (first pass: free)
       bool ok = true;
-      for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+      for (int y = 0, item; ok && (item = item_at(y)) < p.n_items; ++y) {
         int b, hkv, split, T, j0, nk;
         geometry(item, b, hkv, split, T, j0, nk);
         if (T == 0) continue;
@@ -331,22 +347,22 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     // run these loops with identical values; MMAs, commits and TMA loads are issued by one elected lane.
     const uint32_t leader = elect_one();
     // cursor over (non-empty item, tile) in processing order; g = global tile number
-    struct Cur { int item, ne, t, T, b, hkv, j0, g; bool valid; };
+    struct Cur { int y, ne, t, T, b, hkv, j0, g; bool valid; };
     auto first_item = [&](Cur& c, int from, int ne, int g) {
       c.valid = false;
       c.g = g;
-      for (int item = from; item < p.n_items; item += gridDim.x) {
+      for (int y = from, item; (item = item_at(y)) < p.n_items; ++y) {
         int b, hkv, split, T, j0, nk;
         geometry(item, b, hkv, split, T, j0, nk);
-        if (T > 0) { c.item = item; c.ne = ne; c.t = 0; c.T = T; c.b = b; c.hkv = hkv; c.j0 = j0; c.valid = true; return; }
+        if (T > 0) { c.y = y; c.ne = ne; c.t = 0; c.T = T; c.b = b; c.hkv = hkv; c.j0 = j0; c.valid = true; return; }
       }
     };
     auto advance = [&](Cur& c) {
       if (c.t + 1 < c.T) { ++c.t; ++c.g; return; }
-      first_item(c, c.item + gridDim.x, c.ne + 1, c.g + 1);
+      first_item(c, c.y + 1, c.ne + 1, c.g + 1);
     };
     Cur c;
-    first_item(c, blockIdx.x, 0, 0);
+    first_item(c, 0, 0, 0);
     bool ok = true;
     if (warp == 1) {
       // ---- S^T = K Q^T of every tile: its score buffer (g & 3) is free once the softmax group has read tile g - 4
@@ -489,23 +505,23 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
       // of 8-key core matrices 128 bytes apart (so that a softmax thread writes its key's values as one vector store)
       const uint64_t dP0 = make_smem_desc(smem_u32(sP), 128, 2048) & ~((uint64_t)7 << 61);
       // cursor over (non-empty item, tile) in processing order; g = global tile number
-      struct Cur { int item, ne, t, T, b, hkv, j0, g; bool valid; };
+      struct Cur { int y, ne, t, T, b, hkv, j0, g; bool valid; };
       auto first_item = [&](Cur& c, int from, int ne, int g) {
         c.valid = false;
         c.g = g;
-        for (int item = from; item < p.n_items; item += gridDim.x) {
+        for (int y = from, item; (item = item_at(y)) < p.n_items; ++y) {
           int b, hkv, split, T, j0, nk;
           geometry(item, b, hkv, split, T, j0, nk);
-          if (T > 0) { c.item = item; c.ne = ne; c.t = 0; c.T = T; c.b = b; c.hkv = hkv; c.j0 = j0; c.valid = true; return; }
+          if (T > 0) { c.y = y; c.ne = ne; c.t = 0; c.T = T; c.b = b; c.hkv = hkv; c.j0 = j0; c.valid = true; return; }
         }
       };
       auto advance = [&](Cur& c) {
         if (c.t + 1 < c.T) { ++c.t; ++c.g; return; }
-        first_item(c, c.item + gridDim.x, c.ne + 1, c.g + 1);
+        first_item(c, c.y + 1, c.ne + 1, c.g + 1);
       };
       auto ready = [&](uint64_t* bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_test_wait(bar, parity)); };
       Cur cq, cv, cp;                            // next tile to score, to take the vote of, to accumulate
-      first_item(cq, blockIdx.x, 0, 0);
+      first_item(cq, 0, 0, 0);
       cv = cq; cp = cq;
       int kc = 0; uint32_t kpar = 0;             // K ring consumer
       int vi = 0; uint32_t vipar = 1;            // V ring producer side (MALA: copies issued here)
@@ -701,7 +717,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
       pend = false;
       return true;
     };
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+    for (int y = 0, item; ok && (item = item_at(y)) < p.n_items; ++y) {
       int b, hkv, split, T, j0, nk;
       geometry(item, b, hkv, split, T, j0, nk);
       // L of a row = the keys it sees: all nk of the sequence for the newest token, one less per token before it

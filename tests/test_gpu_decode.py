@@ -140,6 +140,23 @@ def _run_paged(mala, oracle, w, tau, num_splits, page_size, seqlens, seed=0, rou
     return dict(skipped=skipped, retained=retained)
 
 
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("B,Nk,S,d,page", [
+    (64, 1024, 8, 128, 16),     # several rounds of items per CTA, short and empty sequences, tiles of several pages
+    (37, 1152, 3, 128, 128),    # a partial last round; partial splits of one, two and three tiles
+    (600, 256, 2, 64, 128),     # more sequences than the ordered list takes: items in the order of their numbers
+    (130, 512, 2, 256, 128),    # 256 columns
+])
+def test_decode_paged_ragged_lengths_in_every_order(mala, oracle, fp8, B, Nk, S, d, page):
+    if fp8 and d == 256:
+        pytest.skip("8-bit caches take head sizes up to 128")
+    rng = np.random.default_rng(B)
+    lens = [int(x) for x in rng.integers(0, Nk + 1, B)]
+    lens[0], lens[1], lens[2] = Nk, 0, 1
+    w = W.custom_decode(B, 4, 2, Nk, d, S, seed=B)
+    (_run_fp8_paged if fp8 else _run_paged)(mala, oracle, w, 1e-4, S, page, lens, seed=B)
+
+
 @pytest.mark.parametrize("tau", [0.0, 1e-4])
 @pytest.mark.parametrize("Nk,S,Hq,Hkv,page,lens", [
     (1024, 4, 8, 2, 128, None),                        # one tile per page, every sequence full
