@@ -4,6 +4,7 @@
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
+#include <atomic>
 #include <mutex>
 
 #include <nvtx3/nvToolsExt.h>
@@ -65,6 +66,15 @@ static int current_device_checked(int* dev_out) {
 template <typename K>
 static bool set_smem(K kernel, int bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+}
+
+// SMs of a device, asked for once.
+static int sm_count(int dev) {
+  static std::atomic<int> known[64];
+  int n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+    known[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // One-time per-device set-up: status word address and dynamic shared memory limits.
@@ -167,11 +177,11 @@ struct ApiScope {
 
 static const float kLog2e = 1.4426950408889634f;
 
-// Forward (prefill) launch: two query blocks per CTA (one with D = 256).
+// Forward (prefill) launch: two query blocks per CTA (one with D = 256 or p.single).
 template <int D, bool kDense>
 static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& p,
                       cudaStream_t stream) {
-  dim3 grid(FwdCfg<D, kDense>::kOne ? p.Tr : (p.Tr + 1) / 2, p.Hq, p.B * (p.num_splits > 1 ? p.num_splits : 1));
+  dim3 grid(FwdCfg<D, kDense>::kOne || p.single ? p.Tr : (p.Tr + 1) / 2, p.Hq, p.B * (p.num_splits > 1 ? p.num_splits : 1));
   if (p.ppt > 1)
     mala_fwd_kernel<D, kDense, true><<<grid, FwdCfg<D, kDense>::kThreads, FwdCfg<D, kDense>::kSmemBytes, stream>>>(tq, tk, tv, p);
   else
@@ -350,6 +360,11 @@ static int fwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse,
   }
   p.scale_log2 = scale * kLog2e;
   p.log2_tau = tau > 0.f ? log2f(tau) : -INFINITY;
+  // Where every query block can have an SM of its own, it gets one: the call then takes as long as its longest block, and
+  // a block alone walks its tiles faster than two that share a CTA (1024 tokens, 2 heads of 64 columns: 17.3 us instead of
+  // 21.0; 512 tokens, 32 heads of 128: 14.1 instead of 17.5).
+  // Beyond that two blocks per CTA share the K tiles and hide one another's softmax.
+  p.single = (long long)p.Tr * Hq * B * num_splits <= sm_count(dev);
   if (p.bitmask) {
     if (cudaMemsetAsync(p.bitmask, 0, (size_t)B * Hq * p.Tr * p.words * sizeof(uint32_t), stream) != cudaSuccess)
       return MALA_ERR_CUDA;
@@ -412,7 +427,7 @@ static int bwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin dou
   int* status = nullptr;
   MALA_TRY(device_setup(dev, &status));
   return bwd_launch(q, k, v, o, dout, lse, dq, dk, dv, st, B0, Hq, Hkv, N0, Nk0, d, causal ? 1 : 0, scale, tau, ws,
-                    ws_bytes, status, (cudaStream_t)cuda_stream, cu, total, cu_k, total_k);
+                    ws_bytes, status, sm_count(dev), (cudaStream_t)cuda_stream, cu, total, cu_k, total_k);
 }
 
 int mala_fwd_chunk_split(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse, const mala_stats* st, int B,

@@ -907,7 +907,7 @@ inline int bwd_launch_scout(const CUtensorMap& tq, const CUtensorMap& tk, const 
 
 inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin dout, const float* lse, mala_tout dq,
                       mala_tout dk, mala_tout dv, const mala_stats* st, int B, int Hq, int Hkv, int N, int Nk, int d,
-                      int causal, float scale, float tau, void* ws, size_t ws_bytes, int* status, cudaStream_t stream,
+                      int causal, float scale, float tau, void* ws, size_t ws_bytes, int* status, int sms, cudaStream_t stream,
                       const int* cu = nullptr, int total = 0, const int* cu_k = nullptr, int total_k = 0) {
   // Packed sequences (cu): N = Nk = the longest sequence; the tensors are [1, total, H, d]; the per-query vectors and
   // the dQ accumulator are laid out per head over Np = total + 128 B rows (rounded up to a tile).
@@ -966,7 +966,12 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
   // kernel that tests and works tile by tile.
   const int wpad = bwd_mask_wpad(T);
   const size_t base_bytes = bwd_align256((size_t)Bl * Hq * Np * D * sizeof(float)) + 3 * vbytes;
-  const bool two_pass = !dense && MALA_BWD_TWO_PASS && (Hq / Hkv) * 2 * wpad <= kScoutMaskWords && (Hq / Hkv) <= 16 &&
+  // A small call (every key block has an SM, and at most sixteen tiles to walk) is a matter of latency: one kernel that
+  // tests as it goes is over before the first pass and the two launches behind it would be, whatever is skipped
+  // (whole backward, 1024 tokens, 2 heads of 64 columns: 27.7 us instead of 39.8, 29.9 instead of 42.2 with 128 columns and
+  // nearly every tile skipped; 512 tokens, 32 / 8 heads: 61 instead of 87).
+  const bool brief = (long long)Tk * Hkv * B <= sms && (Hq / Hkv) * T <= 16;
+  const bool two_pass = !dense && !brief && MALA_BWD_TWO_PASS && (Hq / Hkv) * 2 * wpad <= kScoutMaskWords && (Hq / Hkv) <= 16 &&
                         ws_bytes >= base_bytes + bwd_list_bytes(B, Hq, T, Tk);
   int rc;
   if (two_pass) {

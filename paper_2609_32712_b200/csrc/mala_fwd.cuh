@@ -1,4 +1,5 @@
-// MALA forward (Algorithm 1) for sm_100a, prefill version: two query blocks per CTA (one with a head size above 128).
+// MALA forward (Algorithm 1) for sm_100a, prefill version: two query blocks per CTA (one with a head size above 128, and
+// where there is an SM for every query block).
 //
 // One CTA owns the two consecutive 128-row query blocks A = 2c and B = 2c+1 of one (batch, query
 // head).  They share the K tiles; each block has its own UMMA-issuing warp, softmax warpgroup,
@@ -58,6 +59,7 @@ struct FwdParams {
   // log-normalizer of the range; a merge kernel combines the ranges.
   int num_splits, tps;
   float* o_part;                 // [B, Hq, num_splits, N, D]
+  int single;                    // one query block per CTA instead of two
   int d;                         // head size of the tensors (<= D; the columns d .. D-1 are zeros and never stored)
   float* lse_part;               // [B, Hq, num_splits, N] natural log
   float scale_log2;              // scale * log2(e)
@@ -140,11 +142,12 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int Tr = p.cu ? (Nq + qshift + 127) / 128 : p.Tr;
   const int Tk = p.cu ? (Nkeys + 127) / 128 : p.Tk;
   const int bz = p.cu ? 0 : b;                        // outermost TMA coordinate
-  const int npairs = kOne ? Tr : (Tr + 1) / 2;
+  const bool one = kOne || p.single;
+  const int npairs = one ? Tr : (Tr + 1) / 2;
   if ((int)blockIdx.x >= npairs) return;             // (a sequence shorter than the longest one)
   const int c = npairs - 1 - (int)blockIdx.x;        // longest pairs first
-  int iA = kOne ? c : 2 * c, iB = kOne ? c : 2 * c + 1;
-  bool hasB = !kOne && iB < Tr;
+  int iA = one ? c : 2 * c, iB = one ? c : 2 * c + 1;
+  bool hasB = !one && iB < Tr;
   int dA = p.causal ? iA + koff : Tk - 1;            // newest key block with a legal key, per block
   const int dB = p.causal ? iB + koff : Tk - 1;
   int jlo = 0, jhi = Tk - 1;                         // key blocks of this CTA

@@ -70,6 +70,14 @@ def test_bwd_small_shapes_literal(mala, oracle, N, d, Hq, Hkv, tau):
     _run_isolated(mala, oracle, w, tau)
 
 
+@pytest.mark.parametrize("tau", [1e-4, 1e-2])
+@pytest.mark.parametrize("N,d,Hq,Hkv", [(300, 128, 49, 49), (300, 128, 50, 50), (512, 64, 8, 2), (513, 64, 8, 2)])
+def test_bwd_one_or_two_passes(mala, oracle, N, d, Hq, Hkv, tau):
+    # key blocks for as many SMs as the GPU has and just more of them; sixteen tiles per key block and more
+    w = W.custom_prefill(1, Hq, Hkv, N, d, seed=N + Hq, preset="R")
+    _run_isolated(mala, oracle, w, tau)
+
+
 @pytest.mark.parametrize("tau", [1e-5, 1e-4, 1e-3, 1.0])
 @pytest.mark.parametrize("N,d", [(1024, 128), (1000, 128), (1024, 64)])
 def test_bwd_skipping_regime(mala, oracle, N, d, tau):

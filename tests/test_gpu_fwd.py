@@ -61,6 +61,14 @@ def test_fwd_small_shapes_literal(mala, oracle, N, d, Hq, Hkv, tau):
     _run_and_check(mala, oracle, w, tau)
 
 
+@pytest.mark.parametrize("tau", [0.0, 1e-3])
+@pytest.mark.parametrize("N,d,H", [(130, 64, 74), (130, 64, 75), (300, 128, 49), (300, 128, 50)])
+def test_fwd_one_or_two_blocks_per_cta(mala, oracle, N, d, H, tau):
+    # as many query blocks as a GPU of 148 SMs has SMs (a CTA each), and just more of them (two per CTA)
+    w = W.custom_prefill(1, H, H, N, d, seed=N + H, preset="R")
+    _run_and_check(mala, oracle, w, tau)
+
+
 @pytest.mark.parametrize("tau", [1e-5, 1e-4, 1e-3, 1.0])
 @pytest.mark.parametrize("N,d", [(1024, 128), (1000, 128), (1024, 64)])
 def test_fwd_skipping_regime(mala, oracle, N, d, tau):
