@@ -365,6 +365,8 @@ static int fwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse,
   // 21.0; 512 tokens, 32 heads of 128: 14.1 instead of 17.5).
   // Beyond that two blocks per CTA share the K tiles and hide one another's softmax.
   p.single = (long long)p.Tr * Hq * B * num_splits <= sm_count(dev);
+  p.by_size = order_by_size(4ll * d * Hkv * (pg ? (long long)pg->num_pages * pg->page_size : (long long)Bt * Nkt),
+                            (long long)p.Tr * Hq * B * num_splits);
   if (p.bitmask) {
     if (cudaMemsetAsync(p.bitmask, 0, (size_t)B * Hq * p.Tr * p.words * sizeof(uint32_t), stream) != cudaSuccess)
       return MALA_ERR_CUDA;

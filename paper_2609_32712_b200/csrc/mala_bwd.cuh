@@ -86,6 +86,7 @@ struct BwdParams {
   const uint32_t* sel_rows;    // [B,Hq,Tk] or null (all heads)
   int accum_dkv;
   float scale, scale_log2;
+  int by_size;          // see block_place
 };
 
 template <int D>
@@ -150,7 +151,8 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   __shared__ int early_exit;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int j = blockIdx.x, hkv = blockIdx.y, b = blockIdx.z;
+  const BlockPlace place = block_place(p.by_size);
+  const int j = place.x, hkv = place.y, b = place.z;
   const int G = p.Hq / p.Hkv;
   // this sequence: first row in the tensors, rows, blocks, first row in the padded per-head arrays
   const int row0 = p.cu ? __ldg(p.cu + b) : 0;
@@ -948,6 +950,7 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
   p.cu = cu; p.cu_k = cu_k; p.d = d;
   if (cu_k) { p.koff = 0; p.qshift = 0; }    // per sequence, on the device
   p.scale = scale; p.scale_log2 = scale * 1.4426950408889634f;
+  p.by_size = order_by_size(4ll * d * Hq * Bl * Nt, (long long)Tk * Hkv * B);
   p.list_mask = nullptr; p.wpad = 0; p.sel_rows = nullptr; p.accum_dkv = 0;
   if (p.bitmask &&
       cudaMemsetAsync(p.bitmask, 0, (size_t)B * Hq * Tk * p.words * sizeof(uint32_t), stream) != cudaSuccess)
@@ -986,6 +989,7 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
     sp.Nk = Nk; sp.Tk = Tk; sp.koff = p.koff; sp.qshift = p.qshift; sp.cu = cu; sp.cu_k = cu_k;
     sp.scale_log2 = p.scale_log2;
     sp.sample = MALA_BWD_SAMPLE;
+    sp.by_size = p.by_size;
     CUtensorMap tq2;   // the queries again, in boxes of two tiles
     if (!make_tensor_map_bnhd(&tq2, q.p, Bl, Nt, Hq, d, q.sb, q.sn, q.sh, 256)) return MALA_ERR_TENSOR_MAP;
     rc = (D == 128) ? bwd_launch_scout<128>(tq2, tk, sp, stream) : bwd_launch_scout<64>(tq2, tk, sp, stream);

@@ -53,6 +53,7 @@ struct ScoutParams {
   const int* cu_k;
   int sample;                 // sample the rows first and leave the ones that retain everything to the one-pass kernel
   float scale_log2;
+  int by_size;                // see block_place
 };
 
 template <int D>
@@ -107,7 +108,8 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_con
   __shared__ int early_exit;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ja = 2 * (int)blockIdx.x, jb = ja + 1, hkv = blockIdx.y, b = blockIdx.z;
+  const BlockPlace place = block_place(p.by_size);
+  const int ja = 2 * place.x, jb = ja + 1, hkv = place.y, b = place.z;
   const int G = p.Hq / p.Hkv;
   // this sequence (the geometry of mala_bwd_kernel)
   const int row0 = p.cu ? __ldg(p.cu + b) : 0;

@@ -60,6 +60,7 @@ struct FwdParams {
   int num_splits, tps;
   float* o_part;                 // [B, Hq, num_splits, N, D]
   int single;                    // one query block per CTA instead of two
+  int by_size;                   // see block_place
   int d;                         // head size of the tensors (<= D; the columns d .. D-1 are zeros and never stored)
   float* lse_part;               // [B, Hq, num_splits, N] natural log
   float scale_log2;              // scale * log2(e)
@@ -105,9 +106,10 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int G = p.Hq / p.Hkv;
-  const int sp = p.num_splits > 1 ? (int)blockIdx.z % p.num_splits : 0;
-  const int b = p.num_splits > 1 ? (int)blockIdx.z / p.num_splits : (int)blockIdx.z;
-  const int h = blockIdx.y, hkv = h / G;
+  const BlockPlace place = block_place(p.by_size);
+  const int sp = p.num_splits > 1 ? place.z % p.num_splits : 0;
+  const int b = p.num_splits > 1 ? place.z / p.num_splits : place.z;
+  const int h = place.y, hkv = h / G;
   // this sequence: first rows in the tensors, rows, keys, blocks
   const int row0 = p.cu ? __ldg(p.cu + b) : 0;
   const int Nq = p.cu ? __ldg(p.cu + b + 1) - row0 : p.N;
@@ -144,8 +146,9 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int bz = p.cu ? 0 : b;                        // outermost TMA coordinate
   const bool one = kOne || p.single;
   const int npairs = one ? Tr : (Tr + 1) / 2;
-  if ((int)blockIdx.x >= npairs) return;             // (a sequence shorter than the longest one)
-  const int c = npairs - 1 - (int)blockIdx.x;        // longest pairs first
+  // longest pairs first: of this head and sequence, or (by_size) of all of them, the longest sequence's last pair in front
+  const int c = (p.by_size ? (int)gridDim.x : npairs) - 1 - place.x;
+  if (c < 0 || c >= npairs) return;                  // (a sequence shorter than the longest one)
   int iA = one ? c : 2 * c, iB = one ? c : 2 * c + 1;
   bool hasB = !one && iB < Tr;
   int dA = p.causal ? iA + koff : Tk - 1;            // newest key block with a legal key, per block
