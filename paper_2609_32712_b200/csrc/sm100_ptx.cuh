@@ -123,11 +123,12 @@ __device__ __forceinline__ BlockPlace block_place(int by_size) {
   return {(int)x, (int)(r - z * gridDim.y), (int)z};
 }
 // The rule: by size where what the blocks of different heads share only among themselves (`bytes`: K and V in the forward, Q
-// and dO in the backward) stays in the 126 MB L2 with room to spare; beyond that the heads in flight at a time should be
-// few.  (With that much work a launch has many rounds of blocks and its end matters little: 1 % at 32768 tokens x 32 heads;
-// at 8192 x 16 the busiest SM had 1.54 times the mean of the backward's tiles and 1.31 of the forward's, by size 1.13 and
-// 1.04.)
-inline int order_by_size(long long bytes, long long blocks) { return bytes <= (96ll << 20) && blocks < (1ll << 31); }
+// and dO in the backward) takes up to half of the 126 MB L2; beyond that the heads in flight at a time should be few (by
+// size, a batch of prefill chunks over 411 MB of keys and values took 2366 us instead of 2085, nine packed sequences with
+// 91 and 365 MB 2780 instead of 2730).  With that much work a launch has many rounds of blocks and its end matters little:
+// 1 % at 32768 tokens x 32 heads, whereas at 8192 x 16 the busiest SM had 1.54 times the mean of the backward's tiles and
+// 1.31 of the forward's, by size 1.13 and 1.04 (1385 us for both, by size 1165).
+inline int order_by_size(long long bytes, long long blocks) { return bytes <= (64ll << 20) && blocks < (1ll << 31); }
 
 // ------------------------------------------------------------------------------------------------
 // programmatic dependent launch: a kernel lets its dependents be launched before it has finished; a dependent waits until
