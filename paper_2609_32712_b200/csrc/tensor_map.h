@@ -25,6 +25,15 @@ inline PFN_tensorMapEncodeTiled tensor_map_encoder() {
   return fn;
 }
 
+// Calls the driver's encoder.  It needs a current context, which a thread has only after a runtime call that binds the
+// device's (a backward in an autograd thread whose allocations all came from a cache has made none): bind it and try again.
+template <typename... A>
+inline bool encode_tensor_map(PFN_tensorMapEncodeTiled enc, A... args) {
+  if (enc(args...) == CUDA_SUCCESS) return true;
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess && enc(args...) == CUDA_SUCCESS;
+}
+
 // Tensor map over a bf16 [B, N, H, d] view: coordinates (c, n, h, b), box = 64 columns x box_rows rows,
 // 128-byte swizzle, out-of-range rows read as zero.  Returns false if the driver rejects it
 // (base not 16-byte aligned, a stride not a multiple of 16 bytes, ...).
@@ -44,10 +53,9 @@ inline bool make_tensor_map_bnhd(CUtensorMap* out, const void* base, int B, int 
   cuuint64_t strides[3] = {legal(sn, N), legal(sh, H), legal(sb, B)};
   cuuint32_t box[4] = {64u, (cuuint32_t)box_rows, 1u, 1u};
   cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-  CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
+  return encode_tensor_map(enc, out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // Tensor map over an 8-bit [B, N, H, d] view (strides in elements = bytes): coordinates (c, n, h, b), box = 128 columns
@@ -62,10 +70,9 @@ inline bool make_tensor_map_u8_bnhd(CUtensorMap* out, const void* base, int B, i
   cuuint64_t strides[3] = {legal(sn, N), legal(sh, H), legal(sb, B)};
   cuuint32_t box[4] = {128u, (cuuint32_t)box_rows, 1u, 1u};
   cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-  CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
+  return encode_tensor_map(enc, out, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // Tensor map over the bf16 queries of a decode step, [B, S, H, d]: coordinates (c, h, s, b), box = 64 columns x G
@@ -79,10 +86,9 @@ inline bool make_tensor_map_q_rows(CUtensorMap* out, const void* base, int B, in
   cuuint64_t strides[3] = {legal(sh, H), legal(sn, S), legal(sb, B)};
   cuuint32_t box[4] = {64u, (cuuint32_t)G, (cuuint32_t)S, 1u};
   cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-  CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
+  return encode_tensor_map(enc, out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // Tensor map over fp32 tiles: `ntiles` row-major [128 rows x cols] blocks, `tile_stride_bytes` apart, first one at
@@ -96,10 +102,9 @@ inline bool make_tensor_map_f32_tiles(CUtensorMap* out, const void* base, uint64
   cuuint64_t strides[2] = {(cuuint64_t)cols * 4, (cuuint64_t)tile_stride_bytes};
   cuuint32_t box[3] = {32u, 128u, 1u};
   cuuint32_t estr[3] = {1u, 1u, 1u};
-  CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
+  return encode_tensor_map(enc, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 }  // namespace mala

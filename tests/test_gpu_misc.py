@@ -273,3 +273,27 @@ def test_debug_mode_reports_errors_from_the_call_itself():
     assert r.returncode == 0, r.stderr[-2000:]
     assert "CODE -8" in r.stdout and "DONE" in r.stdout, r.stdout + r.stderr[-1000:]
     assert "[mala debug] mala_decode: device status" in r.stderr
+
+
+def test_first_call_of_a_thread_needs_no_earlier_cuda_call(mala):
+    # a thread that has made no runtime call yet has no current context, which the tensor maps' encoder needs
+    import threading
+    w = W.custom_prefill(1, 2, 2, 256, 64, seed=3)
+    q, k, v = (w[x].cuda() for x in ("q", "k", "v"))
+    o, lse, _ = mala.fwd(q, k, v, w["scale"], 1e-4)
+    o2, lse2, ws = torch.zeros_like(o), torch.zeros_like(lse), torch.empty(256, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    failed = []
+
+    def body():
+        try:
+            mala.fwd(q, k, v, w["scale"], 1e-4, out=o2, lse=lse2, ws=ws)
+        except Exception as e:
+            failed.append(e)
+
+    t = threading.Thread(target=body)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert not failed, failed
+    assert torch.equal(o, o2) and torch.equal(lse, lse2)
