@@ -381,7 +381,8 @@ static int fwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse,
   else rc = dense ? launch_fwd<64, true>(tq, tk, tv, p, stream) : launch_fwd<64, false>(tq, tk, tv, p, stream);
   if (rc != MALA_OK || num_splits == 1) return rc;
   auto merge = D == 256 ? fwd_merge_splits_kernel<256> : D == 128 ? fwd_merge_splits_kernel<128> : fwd_merge_splits_kernel<64>;
-  return launch_dependent(merge, dim3((N + 7) / 8, B * Hq), dim3(256), stream, p.o_part, p.lse_part, p.o, p.o_sb, p.o_sn, p.o_sh,
+  // (all rows in the grid's first coordinate: the others end at 65535, and B * Hq does not)
+  return launch_dependent(merge, dim3((unsigned)((long long)((N + 7) / 8) * B * Hq)), dim3(256), stream, p.o_part, p.lse_part, p.o, p.o_sb, p.o_sn, p.o_sh,
                           lse, Hq, N, num_splits, p.tps, p.Tk, p.koff, p.qshift, p.causal, d) == cudaSuccess
              ? MALA_OK : MALA_ERR_CUDA;
 }

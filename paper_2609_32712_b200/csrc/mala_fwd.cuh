@@ -668,7 +668,8 @@ fwd_merge_splits_kernel(const float* __restrict__ o_part, const float* __restric
                         float* __restrict__ lse, int Hq, int N, int num_splits, int tps, int Tk, int koff, int qshift,
                         int causal, int d) {
   constexpr int L4 = D / 4, V = L4 > 32 ? L4 / 32 : 1;   // float4 per partial; per lane
-  const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y, h = bh % Hq, b = bh / Hq;
+  const int per = (N + 7) / 8, bh = blockIdx.x / per, h = bh % Hq, b = bh / Hq;   // blocks of eight rows per (b, head)
+  const int lane = threadIdx.x & 31, row = (blockIdx.x - bh * per) * 8 + (threadIdx.x >> 5);
   if (row >= N) return;
   const int newest = causal ? (row + qshift) / 128 + koff : Tk - 1;
   const int ns = min(num_splits, newest / tps + 1);

@@ -311,3 +311,22 @@ def test_chunk_split_of_one_range_equals_the_unsplit_call(mala):
     o1, l1, _ = mala.fwd_chunk(q[:, 1024:], k, v, w["scale"], 1e-4)
     o2, l2, _ = mala.fwd_chunk_split(q[:, 1024:], k, v, w["scale"], 1e-4, 1)
     assert torch.equal(o1, o2) and torch.equal(l1, l2)
+
+
+@pytest.mark.parametrize("Nq", [1, 3])
+def test_chunk_split_of_more_heads_and_sequences_than_a_grid_has_rows(mala, Nq):
+    # B * Hq = 65600: more than the second and third coordinate of a grid hold
+    B, Hq, Hkv, Nk, d, S = 1025, 64, 1, 256, 64, 2
+    g = torch.Generator(device="cuda").manual_seed(Nq)
+    q, k, v = (torch.randn((B, n, h, d), generator=g, device="cuda").to(torch.bfloat16) for n, h in ((Nq, Hq), (Nk, Hkv), (Nk, Hkv)))
+    scale = d ** -0.5
+    o, lse, _ = mala.fwd_chunk_split(q, k, v, scale, 0.0, S)
+    torch.cuda.synchronize()
+    assert mala.device_status() == 0
+    s = torch.einsum("bqhd,bkd->bhqk", q.float(), k[:, :, 0].float()) * scale
+    keys = torch.arange(Nk, device="cuda")
+    s.masked_fill_(keys[None, :] > Nk - Nq + torch.arange(Nq, device="cuda")[:, None], -torch.inf)
+    p = torch.softmax(s, -1)
+    ref, a = (torch.einsum("bhqk,bkd->bqhd", p, x) for x in (v[:, :, 0].float(), v[:, :, 0].float().abs()))
+    parity.check_output(o.float().cpu().numpy(), ref.cpu().numpy(), a_ref=a.cpu().numpy())
+    assert (lse - torch.logsumexp(s, -1)).abs().max() <= parity.LSE_ABS
