@@ -137,7 +137,8 @@ inline int order_by_size(long long bytes, long long blocks) { return bytes <= (6
 __device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launches `kernel`, which begins with wait_for_primary(), as a programmatic dependent of the kernel before it.
+// Launches `kernel`, which begins with wait_for_primary(), as a programmatic dependent of the kernel before it.  A launch that
+// fails is reported here alone: the runtime's last error is taken back, so that the next call's check does not meet it.
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
   cudaLaunchAttribute at[1];
@@ -146,7 +147,9 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = stream;
   cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
 }
 
 // ------------------------------------------------------------------------------------------------

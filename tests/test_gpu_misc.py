@@ -1,5 +1,8 @@
 """GPU checks beyond plain parity: strided tensor views, run-to-run determinism, tau-monotonic support,
 ragged mid-size shapes in the skipping regime, and error reporting through the binding."""
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -8,6 +11,8 @@ from paper_2609_32712_b200 import workloads as W
 from tests import parity
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -297,3 +302,25 @@ def test_first_call_of_a_thread_needs_no_earlier_cuda_call(mala):
     torch.cuda.synchronize()
     assert not failed, failed
     assert torch.equal(o, o2) and torch.equal(lse, lse2)
+
+
+def test_a_failed_dependent_launch_leaves_no_error_behind(tmp_path):
+    # a grid that no device takes is refused by the runtime: the launch returns the error, and the runtime's last error,
+    # which later calls check after their own launches, stays clear
+    src = tmp_path / "launch.cu"
+    src.write_text("""
+#include <stdio.h>
+#include "sm100_ptx.cuh"
+__global__ void kernel(int) {}
+int main() {
+  const cudaError_t e = mala::launch_dependent(kernel, dim3(1, 70000, 1), dim3(32), (cudaStream_t)0, 1);
+  const cudaError_t left = cudaGetLastError();
+  printf("%d %d\\n", (int)e, (int)left);
+  return e != cudaSuccess && left == cudaSuccess ? 0 : 1;
+}
+""")
+    exe = str(tmp_path / "launch")
+    subprocess.check_call(["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-o", exe, str(src), "-I",
+                           os.path.join(ROOT, "paper_2609_32712_b200", "csrc")])
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert out.returncode == 0, out.stdout + out.stderr
