@@ -39,7 +39,6 @@ decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ 
   if (lane == 0) red[w] = mx;
   __syncthreads();
   mx = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
-  // (a sequence without keys has no split with mass: its output is 0 and its log-normalizer -inf)
   float Z = 0.f;
   float4 acc[V];
 #pragma unroll
@@ -77,14 +76,17 @@ decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ 
   if (lane == 0) red[w] = Zw;
   __syncthreads();
   Z = (red[0] + red[1]) + (red[2] + red[3]);
-  const float inv = Z > 0.f ? 1.f / Z : 0.f;
+  // (a sequence without keys has no split with mass: its output is 0 and its log-normalizer -inf; so it is with a
+  // normalizer that is not a number, whose sums must not reach the output)
+  const bool any = Z > 0.f;
+  const float inv = any ? 1.f / Z : 0.f;
   for (int c = threadIdx.x; c < d; c += 128) {
     float t = 0.f;
 #pragma unroll
     for (int x = 0; x < 4 * PER; ++x) t += sum[x][c];
-    o[b * o_sb + tok * o_sn + h * o_sh + c] = __float2bfloat16(t * inv);
+    o[b * o_sb + tok * o_sn + h * o_sh + c] = __float2bfloat16(any ? t * inv : 0.f);
   }
-  if (lse_out && threadIdx.x == 0) lse_out[bh] = Z > 0.f ? mx + logf(Z) : -INFINITY;
+  if (lse_out && threadIdx.x == 0) lse_out[bh] = any ? mx + logf(Z) : -INFINITY;
 }
 
 // The merge as a programmatic dependent of the split kernel before it on the stream (which has let it go ahead): its

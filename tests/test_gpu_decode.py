@@ -613,3 +613,20 @@ def test_decode_fp8_small_pages_absent_pages_do_not_set_the_reference(mala, orac
     w["vcache"] = (w["vcache"].float() * 2.0 ** -6).to(torch.bfloat16)
     for tau in (0.0, 1.0):
         _run_fp8_paged(mala, oracle, w, tau, 2, page, [4096, 1497, 48 + page // 2], seed=3)
+
+
+@pytest.mark.parametrize("S", [1, 4, 9])
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_decode_scores_that_are_not_numbers_give_an_empty_result(mala, d, S):
+    # a key that is not a number leaves its KV head's rows without a normalizer: output 0 and log-normalizer -inf, the
+    # values of a sequence without keys; the other heads are untouched
+    w = W.custom_decode(2, 4, 2, 1152, d, S, seed=d + S)
+    q, k, v = (w[x].cuda() for x in ("q", "kcache", "vcache"))
+    o, lse, _ = mala.decode(q, k, v, w["scale"], 0.0, S)
+    k[1, 700, 1, 5] = float("nan")
+    o2, lse2, _ = mala.decode(q, k, v, w["scale"], 0.0, S)
+    torch.cuda.synchronize()
+    assert mala.device_status() == 0
+    assert (o2[1, 0, 2:] == 0).all() and (lse2[1, 2:] == -torch.inf).all()
+    assert torch.equal(o2[0], o[0]) and torch.equal(o2[1, 0, :2], o[1, 0, :2])
+    assert torch.equal(lse2[0], lse[0]) and torch.equal(lse2[1, :2], lse[1, :2])
