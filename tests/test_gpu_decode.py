@@ -615,7 +615,7 @@ def test_decode_fp8_small_pages_absent_pages_do_not_set_the_reference(mala, orac
         _run_fp8_paged(mala, oracle, w, tau, 2, page, [4096, 1497, 48 + page // 2], seed=3)
 
 
-@pytest.mark.parametrize("S", [1, 4, 9])
+@pytest.mark.parametrize("S", [1, 4, 9, 13])
 @pytest.mark.parametrize("d", [64, 128, 256])
 def test_decode_scores_that_are_not_numbers_give_an_empty_result(mala, d, S):
     # a key that is not a number leaves its KV head's rows without a normalizer: output 0 and log-normalizer -inf, the
@@ -630,3 +630,13 @@ def test_decode_scores_that_are_not_numbers_give_an_empty_result(mala, d, S):
     assert (o2[1, 0, 2:] == 0).all() and (lse2[1, 2:] == -torch.inf).all()
     assert torch.equal(o2[0], o[0]) and torch.equal(o2[1, 0, :2], o[1, 0, :2])
     assert torch.equal(lse2[0], lse[0]) and torch.equal(lse2[1, :2], lse[1, :2])
+
+
+@pytest.mark.parametrize("tau", [0.0, 1e-4])
+@pytest.mark.parametrize("S", [2, 5, 12, 13])
+@pytest.mark.parametrize("d", [64, 96, 136, 256])
+def test_decode_merge_of_few_and_more_splits(mala, oracle, d, S, tau):
+    # one warp per row up to twelve splits, a block per row beyond: odd numbers of rows (3 * 5), head sizes between the
+    # kernels' widths, splits without keys (seven tiles)
+    w = W.custom_decode(3, 5, 5, 896, d, S, seed=d + S)
+    _run_and_check(mala, oracle, w, tau, S, rounding_bound=True)
