@@ -253,6 +253,7 @@ inline int decode_launch_with_scratch(mala_tin q, mala_tin kc, mala_tin vc, mala
   p.n_items = B * Hkv * num_splits;
   p.by_splits.set((uint32_t)num_splits);
   p.by_hkv.set((uint32_t)Hkv);
+  p.by_tps.set((uint32_t)p.tps);
   p.scale_log2 = scale * 1.4426950408889634f;
   p.log2_tau = tau > 0.f ? log2f(tau) : -INFINITY;
   if (p.bitmask &&
@@ -264,7 +265,7 @@ inline int decode_launch_with_scratch(mala_tin q, mala_tin kc, mala_tin vc, mala
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return MALA_ERR_CUDA;
   const int grid = p.n_items < sms ? p.n_items : sms;   // persistent: one CTA per SM
-  p.sched = decode_sched_fits(B, p.n_items, grid, 1, D == 256 ? DecCfgT<256>::kSchedItems : DecCfg::kSchedItems);
+  p.sched = p.seqlens && decode_sched_fits(B, p.n_items, grid, 1, D == 256 ? DecCfgT<256>::kSchedItems : DecCfg::kSchedItems);
   const int R = G * Sq;   // rows of a work item
 #define MALA_DEC_LAUNCH3(DENSE, GP, MULTI)                                                                           \
   {                                                                                                                  \
@@ -340,6 +341,7 @@ inline int decode_fp8_launch(mala_tin q, mala_tin kc, mala_tin vc, const float* 
   p.n_items = B * Hkv * num_splits; p.nt = (Nk + 127) / 128;
   p.by_splits.set((uint32_t)num_splits);
   p.by_hkv.set((uint32_t)Hkv);
+  p.by_tps.set((uint32_t)p.tps);
   p.scale_log2 = scale * 1.4426950408889634f;
   p.log2_tau = tau > 0.f ? log2f(tau) : -INFINITY;
   if (p.bitmask &&
@@ -350,7 +352,7 @@ inline int decode_fp8_launch(mala_tin q, mala_tin kc, mala_tin vc, const float* 
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return MALA_ERR_CUDA;
   const int grid = p.n_items < sms ? p.n_items : sms;
-  p.sched = decode_sched_fits(B, p.n_items, grid, 2, DecF8Cfg<2, false>::kSchedItems);   // (two streams)
+  p.sched = p.seqlens && decode_sched_fits(B, p.n_items, grid, 2, DecF8Cfg<2, false>::kSchedItems);   // (two streams)
 #define MALA_F8_LAUNCH(DENSE, GP)                                                                                      \
   do {                                                                                                                  \
     if (Sq > 1) mala_decode_fp8_kernel<DENSE, GP, false, 2, false, true><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p); \

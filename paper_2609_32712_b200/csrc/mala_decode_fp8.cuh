@@ -66,7 +66,7 @@ struct DecF8Params {
   const float* vscale;           // [B, Hkv, nt]
   int B, Hq, Hkv, Nk, tps, num_splits, words, n_items, nt;
   float scale_log2, log2_tau;
-  FastDiv by_splits, by_hkv;
+  FastDiv by_splits, by_hkv, by_tps;
   int sched;                     // items in the order of decode_schedule
   // paged cache (block_table != null): K / V are [num_pages, page_size, Hkv, d], the scales [num_pages, Hkv, tpp];
   // Nk = max_pages * page_size lays out the splits, a sequence holds seqlens[b] keys (null: Nk)
@@ -212,8 +212,8 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     for (int i = tid; i < (2 * Cfg::kQ8Bytes + PP * Cfg::kP8Bytes) / 16; i += Cfg::kThreads)
       reinterpret_cast<uint4*>(sQ8_of(k))[i] = make_uint4(0u, 0u, 0u, 0u);
   if (p.sched)   // (its tables lie in the K ring, which nothing has been copied into yet)
-    decode_schedule<NG, Cfg::kThreads>(sched, reinterpret_cast<int*>(sKr_of(0)), kPaged ? p.seqlens : nullptr, p.B, p.Hkv,
-                                       p.num_splits, p.tps, p.Nk, p.n_items);
+    decode_schedule<NG, Cfg::kThreads>(sched, sKr_of(0), p.seqlens, p.B, p.Hkv, p.by_hkv, p.by_tps, p.num_splits, p.tps, p.Nk,
+                                       p.n_items);
   fence_proxy_async_smem();
   if (tid == 0) {
     early_exit = (*(volatile int*)status != 0);

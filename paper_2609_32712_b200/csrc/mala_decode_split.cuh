@@ -50,7 +50,7 @@ struct DecParams {
   int Sq;                        // new tokens per sequence (the last Sq positions of the cache); rows = Sq * Hq/Hkv
   int B, Hq, Hkv, Nk, tps, num_splits, words, n_items;   // Nk: longest cache the splits are laid out for
   int sched;                     // items in the order of decode_schedule
-  FastDiv by_splits, by_hkv;
+  FastDiv by_splits, by_hkv, by_tps;
   float scale_log2, log2_tau;
 };
 
@@ -165,7 +165,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   // likewise the rows R..15 of the P^T ring, so that those columns of O^T stay finite
   for (int i = tid; i < DecCfg::kPStages * DecCfg::kPBytes / 16; i += DecCfg::kThreads) reinterpret_cast<uint4*>(sP)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (p.sched)   // (its tables lie in the K ring, which nothing has been copied into yet)
-    decode_schedule<1, DecCfg::kThreads>(sched, reinterpret_cast<int*>(sK), p.seqlens, p.B, p.Hkv, p.num_splits, p.tps, p.Nk, p.n_items);
+    decode_schedule<1, DecCfg::kThreads>(sched, sK, p.seqlens, p.B, p.Hkv, p.by_hkv, p.by_tps, p.num_splits, p.tps, p.Nk, p.n_items);
   fence_proxy_async_smem();
   if (tid == 0) {
     early_exit = (*(volatile int*)status != 0);

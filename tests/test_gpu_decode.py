@@ -8,6 +8,9 @@ from tests import parity
 
 pytestmark = pytest.mark.gpu
 
+# lengths of 40 sequences, up to 1024 keys
+RAGGED40 = [1024, 0, 1, 128, 129] + [int(x) for x in np.random.default_rng(40).integers(0, 1025, 35)]
+
 
 @pytest.fixture(scope="module")
 def mala():
@@ -157,6 +160,23 @@ def test_decode_paged_ragged_lengths_in_every_order(mala, oracle, fp8, B, Nk, S,
     (_run_fp8_paged if fp8 else _run_paged)(mala, oracle, w, 1e-4, S, page, lens, seed=B)
 
 
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("B,Nk,S,d,page", [
+    (256, 384, 1, 128, 128),    # as many sequences as the ordered list takes, splits of three tiles,
+    (257, 384, 1, 128, 128),    # and one more
+    (20, 20480, 4, 64, 128),    # splits of 40 tiles: more sizes than the order tells apart
+])
+def test_decode_paged_ragged_lengths_at_the_edges_of_the_order(mala, oracle, fp8, B, Nk, S, d, page):
+    lens = [int(x) for x in np.random.default_rng(B).integers(0, Nk + 1, B)]
+    lens[0], lens[1], lens[2] = Nk, 0, 1
+    w = W.custom_decode(B, 4, 2, Nk, d, S, seed=B)
+    # (short sequences have outputs of the size of their values, so the bf16 run is held to the rounding bound too)
+    if fp8:
+        _run_fp8_paged(mala, oracle, w, 1e-4, S, page, lens, seed=B)
+    else:
+        _run_paged(mala, oracle, w, 1e-4, S, page, lens, seed=B, rounding_bound=True)
+
+
 @pytest.mark.parametrize("tau", [0.0, 1e-4])
 @pytest.mark.parametrize("Nk,S,Hq,Hkv,page,lens", [
     (1024, 4, 8, 2, 128, None),                        # one tile per page, every sequence full
@@ -269,6 +289,8 @@ def test_decode_multi_of_one_token_equals_decode(mala):
 @pytest.mark.parametrize("Nk,S,Hq,Hkv,page,Sq,lens", [
     (2048, 4, 8, 2, 256, 4, [2048, 1000, 129, 3]),     # 16 rows; the last sequence holds fewer keys than new tokens
     (1536, 3, 4, 2, 128, 3, [1536, 1, 700]),
+    (1024, 4, 8, 2, 128, 4, RAGGED40),                 # more work items than SMs: taken by size
+    (1024, 4, 8, 2, 32, 2, RAGGED40),
 ])
 def test_decode_paged_with_several_new_tokens(mala, oracle, Nk, S, Hq, Hkv, page, Sq, lens, tau):
     B = len(lens)
@@ -480,6 +502,8 @@ def _run_fp8_paged(mala, oracle, w, tau, num_splits, page_size, seqlens, seed=0)
     (1536, 3, 4, 1, 32, [1, 1536, 0, 700]),            # pages of 32 keys
     (4096, 16, 16, 2, 64, [4096, 2049, 300]),          # pages of 64 keys, eight heads per KV head
     (1040, 2, 6, 2, 16, [1040, 1025, 17]),             # a table whose last tile is partly past the row's end
+    (1024, 4, 16, 2, 128, RAGGED40),                   # eight heads per KV head, more work items than SMs: taken by size
+    (1024, 4, 10, 2, 16, RAGGED40),                    # five, small pages
 ])
 def test_decode_fp8_paged_literal(mala, oracle, Nk, S, Hq, Hkv, page, lens, tau):
     B = 2 if lens is None else len(lens)
