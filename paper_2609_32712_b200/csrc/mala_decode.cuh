@@ -183,18 +183,28 @@ inline size_t decode_workspace_bytes(int B, int Hq, int d, int S) {   // d: the 
 
 inline bool decode_set_attributes() {
   bool ok = true;
-#define MALA_DEC_ATTR(DENSE, GP, MULTI) \
-  ok = ok && cudaFuncSetAttribute(mala_decode_split_kernel<DENSE, GP, MULTI, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg::kSmemBytes) == cudaSuccess; \
-  ok = ok && cudaFuncSetAttribute(mala_decode_split_kernel<DENSE, GP, MULTI, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg::kSmemBytes) == cudaSuccess; \
-  ok = ok && cudaFuncSetAttribute(mala_decode_split_kernel<DENSE, GP, MULTI, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfgT<256>::kSmemBytes) == cudaSuccess;
-#define MALA_DEC_ATTR_GP(GP) MALA_DEC_ATTR(false, GP, false) MALA_DEC_ATTR(true, GP, false) MALA_DEC_ATTR(false, GP, true) MALA_DEC_ATTR(true, GP, true)
+#define MALA_DEC_ATTR(DENSE, GP, MULTI, SCHED) \
+  ok = ok && cudaFuncSetAttribute(mala_decode_split_kernel<DENSE, GP, MULTI, 128, SCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg::kSmemBytes) == cudaSuccess; \
+  ok = ok && cudaFuncSetAttribute(mala_decode_split_kernel<DENSE, GP, MULTI, 64, SCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg::kSmemBytes) == cudaSuccess; \
+  ok = ok && cudaFuncSetAttribute(mala_decode_split_kernel<DENSE, GP, MULTI, 256, SCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfgT<256>::kSmemBytes) == cudaSuccess;
+#define MALA_DEC_ATTR_S(GP, SCHED) MALA_DEC_ATTR(false, GP, false, SCHED) MALA_DEC_ATTR(true, GP, false, SCHED) MALA_DEC_ATTR(false, GP, true, SCHED) MALA_DEC_ATTR(true, GP, true, SCHED)
+#define MALA_DEC_ATTR_GP(GP) MALA_DEC_ATTR_S(GP, false) MALA_DEC_ATTR_S(GP, true)
   MALA_DEC_ATTR_GP(1) MALA_DEC_ATTR_GP(2) MALA_DEC_ATTR_GP(4) MALA_DEC_ATTR_GP(8) MALA_DEC_ATTR_GP(16)
-#define MALA_F8_ATTR(DENSE, GP) \
-  ok = ok && cudaFuncSetAttribute(mala_decode_fp8_kernel<DENSE, GP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecF8Cfg<2, DENSE>::kSmemBytes) == cudaSuccess && cudaFuncSetAttribute(mala_decode_fp8_kernel<DENSE, GP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecF8Cfg<2, DENSE>::kSmemBytes) == cudaSuccess && cudaFuncSetAttribute(mala_decode_fp8_kernel<DENSE, GP, true, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecF8Cfg<2, DENSE>::kSmemBytes) == cudaSuccess && cudaFuncSetAttribute(mala_decode_fp8_kernel<DENSE, GP, false, 2, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecF8Cfg<2, DENSE>::kSmemBytes) == cudaSuccess;
-  MALA_F8_ATTR(false, 1) MALA_F8_ATTR(true, 1) MALA_F8_ATTR(false, 2) MALA_F8_ATTR(true, 2) MALA_F8_ATTR(false, 4) MALA_F8_ATTR(true, 4)
-  MALA_F8_ATTR(false, 8) MALA_F8_ATTR(true, 8)
+#define MALA_F8_ATTR1(DENSE, ...) \
+  ok = ok && cudaFuncSetAttribute(mala_decode_fp8_kernel<DENSE, __VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize, DecF8Cfg<2, DENSE>::kSmemBytes) == cudaSuccess;
+#define MALA_F8_ATTR(DENSE, GP) MALA_F8_ATTR1(DENSE, GP, false) MALA_F8_ATTR1(DENSE, GP, false, 2, false, true)
+#define MALA_F8_ATTR_S(DENSE, GP, SCHED) \
+  MALA_F8_ATTR1(DENSE, GP, true, 2, false, false, SCHED) MALA_F8_ATTR1(DENSE, GP, true, 2, true, false, SCHED)
+#define MALA_F8_ATTR_GP(GP) \
+  MALA_F8_ATTR(false, GP) MALA_F8_ATTR_S(false, GP, false) MALA_F8_ATTR_S(false, GP, true) \
+  MALA_F8_ATTR(true, GP) MALA_F8_ATTR_S(true, GP, false) MALA_F8_ATTR_S(true, GP, true)
+  MALA_F8_ATTR_GP(1) MALA_F8_ATTR_GP(2) MALA_F8_ATTR_GP(4) MALA_F8_ATTR_GP(8)
+#undef MALA_F8_ATTR_GP
+#undef MALA_F8_ATTR_S
+#undef MALA_F8_ATTR1
 #undef MALA_F8_ATTR
 #undef MALA_DEC_ATTR_GP
+#undef MALA_DEC_ATTR_S
 #undef MALA_DEC_ATTR
   return ok;
 }
@@ -265,23 +275,28 @@ inline int decode_launch_with_scratch(mala_tin q, mala_tin kc, mala_tin vc, mala
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return MALA_ERR_CUDA;
   const int grid = p.n_items < sms ? p.n_items : sms;   // persistent: one CTA per SM
-  p.sched = p.seqlens && decode_sched_fits(B, p.n_items, grid, 1, D == 256 ? DecCfgT<256>::kSchedItems : DecCfg::kSchedItems);
+  const bool sched = p.seqlens && decode_sched_fits(B, p.n_items, grid, 1, D == 256 ? DecCfgT<256>::kSchedItems : DecCfg::kSchedItems);
   const int R = G * Sq;   // rows of a work item
-#define MALA_DEC_LAUNCH3(DENSE, GP, MULTI)                                                                           \
+#define MALA_DEC_LAUNCH3(DENSE, GP, MULTI, SCHED)                                                                           \
   {                                                                                                                  \
-    if (D == 256) mala_decode_split_kernel<DENSE, GP, MULTI, 256><<<grid, DecCfg::kThreads, DecCfgT<256>::kSmemBytes, stream>>>(tq, tk, tv, p); \
-    else if (D == 128) mala_decode_split_kernel<DENSE, GP, MULTI, 128><<<grid, DecCfg::kThreads, DecCfg::kSmemBytes, stream>>>(tq, tk, tv, p); \
-    else mala_decode_split_kernel<DENSE, GP, MULTI, 64><<<grid, DecCfg::kThreads, DecCfg::kSmemBytes, stream>>>(tq, tk, tv, p);           \
+    if (D == 256) mala_decode_split_kernel<DENSE, GP, MULTI, 256, SCHED><<<grid, DecCfg::kThreads, DecCfgT<256>::kSmemBytes, stream>>>(tq, tk, tv, p); \
+    else if (D == 128) mala_decode_split_kernel<DENSE, GP, MULTI, 128, SCHED><<<grid, DecCfg::kThreads, DecCfg::kSmemBytes, stream>>>(tq, tk, tv, p); \
+    else mala_decode_split_kernel<DENSE, GP, MULTI, 64, SCHED><<<grid, DecCfg::kThreads, DecCfg::kSmemBytes, stream>>>(tq, tk, tv, p);           \
   }
-#define MALA_DEC_LAUNCH2(DENSE, GP)          \
-  {                                          \
-    if (Sq > 1) MALA_DEC_LAUNCH3(DENSE, GP, true) \
-    else MALA_DEC_LAUNCH3(DENSE, GP, false)  \
+#define MALA_DEC_LAUNCH2(DENSE, GP, SCHED)            \
+  {                                                   \
+    if (Sq > 1) MALA_DEC_LAUNCH3(DENSE, GP, true, SCHED) \
+    else MALA_DEC_LAUNCH3(DENSE, GP, false, SCHED)    \
   }
-#define MALA_DEC_LAUNCH(GP)            \
-  {                                    \
-    if (tau == 0.f) MALA_DEC_LAUNCH2(true, GP) \
-    else MALA_DEC_LAUNCH2(false, GP)   \
+#define MALA_DEC_LAUNCH1(GP, SCHED)                   \
+  {                                                   \
+    if (tau == 0.f) MALA_DEC_LAUNCH2(true, GP, SCHED) \
+    else MALA_DEC_LAUNCH2(false, GP, SCHED)           \
+  }
+#define MALA_DEC_LAUNCH(GP)                           \
+  {                                                   \
+    if (sched) MALA_DEC_LAUNCH1(GP, true)           \
+    else MALA_DEC_LAUNCH1(GP, false)                  \
   }
   if (R <= 1) MALA_DEC_LAUNCH(1)
   else if (R <= 2) MALA_DEC_LAUNCH(2)
@@ -289,6 +304,7 @@ inline int decode_launch_with_scratch(mala_tin q, mala_tin kc, mala_tin vc, mala
   else if (R <= 8) MALA_DEC_LAUNCH(8)
   else MALA_DEC_LAUNCH(16)
 #undef MALA_DEC_LAUNCH
+#undef MALA_DEC_LAUNCH1
 #undef MALA_DEC_LAUNCH2
 #undef MALA_DEC_LAUNCH3
   if (cudaGetLastError() != cudaSuccess) return MALA_ERR_CUDA;
@@ -352,20 +368,30 @@ inline int decode_fp8_launch(mala_tin q, mala_tin kc, mala_tin vc, const float* 
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return MALA_ERR_CUDA;
   const int grid = p.n_items < sms ? p.n_items : sms;
-  p.sched = p.seqlens && decode_sched_fits(B, p.n_items, grid, 2, DecF8Cfg<2, false>::kSchedItems);   // (two streams)
-#define MALA_F8_LAUNCH(DENSE, GP)                                                                                      \
-  do {                                                                                                                  \
-    if (Sq > 1) mala_decode_fp8_kernel<DENSE, GP, false, 2, false, true><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p); \
-    else if (small) mala_decode_fp8_kernel<DENSE, GP, true, 2, true><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p); \
-    else if (pg) mala_decode_fp8_kernel<DENSE, GP, true><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p); \
-    else mala_decode_fp8_kernel<DENSE, GP, false><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p);  \
+  const bool sched = p.seqlens && decode_sched_fits(B, p.n_items, grid, 2, DecF8Cfg<2, false>::kSchedItems);   // (two streams)
+#define MALA_F8_LAUNCH1(DENSE, GP, ...) \
+  mala_decode_fp8_kernel<DENSE, GP, __VA_ARGS__><<<grid, DecF8Cfg<2, DENSE, (GP > 4)>::kThreads, DecF8Cfg<2, DENSE>::kSmemBytes, stream>>>(tq, tk, tv, p)
+#define MALA_F8_LAUNCH2(DENSE, GP, SCHED)                                  \
+  do {                                                                     \
+    if (Sq > 1) MALA_F8_LAUNCH1(DENSE, GP, false, 2, false, true);         \
+    else if (small) MALA_F8_LAUNCH1(DENSE, GP, true, 2, true, false, SCHED); \
+    else if (pg) MALA_F8_LAUNCH1(DENSE, GP, true, 2, false, false, SCHED); \
+    else MALA_F8_LAUNCH1(DENSE, GP, false);                                \
   } while (0)
-  const bool dense = (tau == 0.f);
-  if (R <= 1) { if (dense) MALA_F8_LAUNCH(true, 1); else MALA_F8_LAUNCH(false, 1); }
-  else if (R <= 2) { if (dense) MALA_F8_LAUNCH(true, 2); else MALA_F8_LAUNCH(false, 2); }
-  else if (R <= 4) { if (dense) MALA_F8_LAUNCH(true, 4); else MALA_F8_LAUNCH(false, 4); }
-  else { if (dense) MALA_F8_LAUNCH(true, 8); else MALA_F8_LAUNCH(false, 8); }
+#define MALA_F8_LAUNCH(GP)                                                 \
+  do {                                                                     \
+    if (tau == 0.f && sched) MALA_F8_LAUNCH2(true, GP, true);              \
+    else if (tau == 0.f) MALA_F8_LAUNCH2(true, GP, false);                 \
+    else if (sched) MALA_F8_LAUNCH2(false, GP, true);                      \
+    else MALA_F8_LAUNCH2(false, GP, false);                                \
+  } while (0)
+  if (R <= 1) MALA_F8_LAUNCH(1);
+  else if (R <= 2) MALA_F8_LAUNCH(2);
+  else if (R <= 4) MALA_F8_LAUNCH(4);
+  else MALA_F8_LAUNCH(8);
 #undef MALA_F8_LAUNCH
+#undef MALA_F8_LAUNCH2
+#undef MALA_F8_LAUNCH1
   if (cudaGetLastError() != cudaSuccess) return MALA_ERR_CUDA;
   return launch_decode_merge(128, B * Sq * Hq, p.o_part, p.lse_part, o, Sq > 1 ? o.sn : 0, lse_opt, Sq, Hq, num_splits, d,
                              stream);

@@ -49,7 +49,6 @@ struct DecParams {
                                  // per page
   int Sq;                        // new tokens per sequence (the last Sq positions of the cache); rows = Sq * Hq/Hkv
   int B, Hq, Hkv, Nk, tps, num_splits, words, n_items;   // Nk: longest cache the splits are laid out for
-  int sched;                     // items in the order of decode_schedule
   FastDiv by_splits, by_hkv, by_tps;
   float scale_log2, log2_tau;
 };
@@ -121,7 +120,12 @@ __device__ __forceinline__ void lds_row(const float* src, float (&dst)[N]) {
 // 64-column panel is filled; O^T is then still accumulated as a 128-row MMA whose rows 64.. (fed from the unfilled
 // half of the V stage) are never read.  With D = 256 O^T is two 128-row MMAs per key step, on the tile's panels 0-1
 // and 2-3, into two accumulators; a softmax thread then owns the output channels kt and 128 + kt.
-template <bool kDense, int GP, bool kMulti, int D>
+// kSched: the CTA takes its items from the list of decode_schedule.  A template parameter, because items that come out of
+// shared memory are not uniform values to the compiler, and neither is anything worked out from them.  With a branch on a
+// launch parameter: 19 sequences of 53645 keys (dense, 64 columns, 64 / 8 heads), which take the order of the numbers, 506 us
+// instead of 498; 4 of 16389 (four tokens, 32 / 8 heads) 84.5 instead of 80.1; 8 of up to 16000 in pages of 16 keys,
+// which take the list, 76.5 instead of 74.4.
+template <bool kDense, int GP, bool kMulti, int D, bool kSched>
 __global__ void __launch_bounds__(384, 1)
 mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                          const __grid_constant__ CUtensorMap tmV, const DecParams p) {
@@ -152,7 +156,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   __shared__ int v_row[8], v_outer[8];     // TMA coordinates of the V tile of tile g (ring; written by the producer;
                                            // pages smaller than a tile: sequence and key block instead)
   __shared__ __align__(16) float xch_max[2][2][4][8], xch_sum[2][2][4][8];   // [buffer][group][warp][row]: per-tile exchange
-  __shared__ uint16_t sched[DecCfg::kSchedItems];   // the CTA's items when p.sched
+  __shared__ uint16_t sched[kSched ? DecCfg::kSchedItems : 1];   // the CTA's items
   __shared__ int early_exit;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -164,7 +168,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   for (int i = tid; i < 2 * DecCfg::kQBytes / 16; i += DecCfg::kThreads) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0u, 0u, 0u, 0u);
   // likewise the rows R..15 of the P^T ring, so that those columns of O^T stay finite
   for (int i = tid; i < DecCfg::kPStages * DecCfg::kPBytes / 16; i += DecCfg::kThreads) reinterpret_cast<uint4*>(sP)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (p.sched)   // (its tables lie in the K ring, which nothing has been copied into yet)
+  if constexpr (kSched)   // (its tables lie in the K ring, which nothing has been copied into yet)
     decode_schedule<1, DecCfg::kThreads>(sched, sK, p.seqlens, p.B, p.Hkv, p.by_hkv, p.by_tps, p.num_splits, p.tps, p.Nk, p.n_items);
   fence_proxy_async_smem();
   if (tid == 0) {
@@ -193,10 +197,10 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   const uint32_t tb = tmem_base_s;
 
   // the CTA's y-th work item (>= n_items: no more)
-  const int n_mine = (p.n_items + (int)gridDim.x - 1) / (int)gridDim.x;
+  [[maybe_unused]] const int n_mine = (p.n_items + (int)gridDim.x - 1) / (int)gridDim.x;
   auto item_at = [&](int y) -> int {
-    if (p.sched) return y < n_mine ? (int)sched[y] : p.n_items;
-    return (int)blockIdx.x + y * (int)gridDim.x;
+    if constexpr (kSched) return y < n_mine ? (int)sched[y] : p.n_items;
+    else return (int)blockIdx.x + y * (int)gridDim.x;
   };
   // geometry of work item `item`: batch, KV head, split, number of legal tiles, newest key block, keys of the sequence.
   // The KV head is the fastest index of an item's number: CTAs side by side then read the same rows of a key-major cache.
