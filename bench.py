@@ -5,10 +5,10 @@ A step is one pass of the whole path -- mala_fwd then mala_bwd at tolerance tau 
 seeded synthetic input of the benchmark definition's 32K configuration (cfg3; --workload selects
 another).  `value` is dense-equivalent TFLOP/s of fwd+bwd (FullAttn FLOP model: 4*B*Hq*N^2*d/2 forward,
 2.5x that backward) with inputs resident in HBM; `e2e` is the same metric with pinned-host inputs copied
-in and results copied out every step.  The line also carries, under `detail`, fwd / bwd latency of the
-MALA and dense kernels on cfg3 / cfg4 (literal and paper-regime "R" inputs), decode latency on cfg5
-(literal and gated "D" inputs), the skipped-tile fractions, and for cfg3 R and cfg5 D the work / fidelity
-figures (retained slots, omitted mass, relative L2 against the dense path) at tau = 1e-4, 1e-2 and 1.
+in and results copied out every step.  The file that the line names as `detail_file` (--detail-file; many times the line's
+length, so not part of it) holds the fwd / bwd latency of the MALA and dense kernels on cfg3 / cfg4 (literal and
+paper-regime "R" inputs), decode latency on cfg5 (literal and gated "D" inputs), the skipped-tile fractions, and for cfg3 R and
+cfg5 D the work / fidelity figures (retained slots, omitted mass, relative L2 against the dense path) at tau = 1e-4, 1e-2 and 1.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
   python bench.py --only fwd|bwd|decode|decode8 --workload cfg2 --preset R --tau 1e-4 --iters 3
@@ -584,6 +584,15 @@ def run_only(args, dev):
     print("ok")
 
 
+def result_line(out, detail, path):
+    """The one line of a run as JSON; the detail table goes to the file `path`, which the line names."""
+    if detail:
+        with open(path, "w") as f:
+            json.dump(detail, f, indent=1)
+        out = dict(out, detail_file=os.path.relpath(path, ROOT))
+    return json.dumps(out)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -604,6 +613,7 @@ def main():
                          "as the decode rows always do) and the secondary rows (chunks, packed sequences, head types "
                          "...) 3 + 20; config.protocol in the output says which")
     ap.add_argument("--no-detail", action="store_true", help="skip the per-config detail table")
+    ap.add_argument("--detail-file", default=os.path.join(ROOT, "bench_detail.json"), help="where the detail table goes")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 0)
@@ -1076,11 +1086,11 @@ def main():
         "fwd_ms": fwd_ms, "bwd_ms": bwd_ms,
         "fwd_retained_frac": ts["fwd_retained"] / ts["fwd_legal"], "bwd_retained_frac": ts["bwd_retained"] / ts["bwd_legal"],
         "clocks": clocks, "e2e": e2e, "gpu_launches": (6 if tau > 0 else 4) * args.steps,   # (timed region per step: fwd + preprocess, main kernel(s) -- three at tau > 0 -- and dQ convert of the backward)
-        "roofline": roofline, "cpu_baseline": cpu_baseline, "detail": detail,
+        "roofline": roofline, "cpu_baseline": cpu_baseline,
     }
     if tp8 is not None:
         out["tp8"] = tp8
-    print(json.dumps(out))
+    print(result_line(out, detail, args.detail_file))
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()

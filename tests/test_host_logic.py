@@ -206,6 +206,18 @@ def test_flop_model_matches_the_papers_accounting():
     assert bench.whole_job_value(1e12, 4, 1000.0) == pytest.approx(4.0)
 
 
+def test_bench_line_stays_short_and_names_the_detail_file(tmp_path):
+    sys.path.insert(0, ROOT)
+    import bench
+    path = str(tmp_path / "detail.json")
+    detail = {f"row{i}": {"us": float(i)} for i in range(1000)}
+    line = bench.result_line({"metric": "m", "value": 1.0}, detail, path)
+    assert len(line) < 1000 and json.loads(line)["value"] == 1.0
+    assert json.load(open(path)) == detail
+    assert os.path.realpath(os.path.join(ROOT, json.loads(line)["detail_file"])) == os.path.realpath(path)
+    assert json.loads(bench.result_line({"value": 2.0}, {}, path)) == {"value": 2.0}
+
+
 def _gloo_worker(rank, world, port, q):
     os.environ.update(MASTER_ADDR="127.0.0.1", MASTER_PORT=str(port), RANK=str(rank), WORLD_SIZE=str(world))
     import torch.distributed as dist
