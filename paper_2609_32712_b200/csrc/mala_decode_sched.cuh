@@ -14,7 +14,8 @@
 
 namespace mala {
 
-// Division of a 32-bit number by a divisor known at launch, as a multiplication and shifts (every role works out for
+// Division of a 32-bit number by a divisor known at launch, as a multiplication and shifts (Granlund and Montgomery's
+// round-up method for an invariant divisor; every role works out for
 // itself which sequence, KV head and split a work item is; hardware has no integer divide, and the few dozen
 // dependent instructions of an emulated one would sit on the per-tile chain of the softmax threads).
 struct FastDiv {
