@@ -365,8 +365,12 @@ static int fwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse,
   // 21.0; 512 tokens, 32 heads of 128: 14.1 instead of 17.5).
   // Beyond that two blocks per CTA share the K tiles and hide one another's softmax.
   p.single = (long long)p.Tr * Hq * B * num_splits <= sm_count(dev);
-  p.by_size = order_by_size(4ll * d * Hkv * (pg ? (long long)pg->num_pages * pg->page_size : (long long)Bt * Nkt),
-                            (long long)p.Tr * Hq * B * num_splits);
+  // (pages: at most the ones that the block tables can name, however large the pool is)
+  const long long keys = pg ? (long long)(pg->num_pages < (long long)B * pg->max_pages_per_seq
+                                              ? pg->num_pages : (long long)B * pg->max_pages_per_seq) * pg->page_size
+                            : (long long)Bt * Nkt;
+  const long long blocks = (long long)(p.single || D == 256 ? p.Tr : (p.Tr + 1) / 2) * Hq * B * num_splits;
+  p.by_size = order_by_size(4ll * d * Hkv * keys, 72ll << 20, blocks, sm_count(dev), N, Nk);
   if (p.bitmask) {
     if (cudaMemsetAsync(p.bitmask, 0, (size_t)B * Hq * p.Tr * p.words * sizeof(uint32_t), stream) != cudaSuccess)
       return MALA_ERR_CUDA;

@@ -950,7 +950,7 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
   p.cu = cu; p.cu_k = cu_k; p.d = d;
   if (cu_k) { p.koff = 0; p.qshift = 0; }    // per sequence, on the device
   p.scale = scale; p.scale_log2 = scale * 1.4426950408889634f;
-  p.by_size = order_by_size(4ll * d * Hq * Bl * Nt, (long long)Tk * Hkv * B);
+  p.by_size = order_by_size(4ll * d * Hq * Bl * Nt, 192ll << 20, (long long)Tk * Hkv * B, sms, N, Nk);
   p.list_mask = nullptr; p.wpad = 0; p.sel_rows = nullptr; p.accum_dkv = 0;
   if (p.bitmask &&
       cudaMemsetAsync(p.bitmask, 0, (size_t)B * Hq * Tk * p.words * sizeof(uint32_t), stream) != cudaSuccess)

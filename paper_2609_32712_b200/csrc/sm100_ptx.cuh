@@ -122,13 +122,21 @@ __device__ __forceinline__ BlockPlace block_place(int by_size) {
   const uint32_t x = at / n, r = at - x * n, z = r / gridDim.y;
   return {(int)x, (int)(r - z * gridDim.y), (int)z};
 }
-// The rule: by size where what the blocks of different heads share only among themselves (`bytes`: K and V in the forward, Q
-// and dO in the backward) takes up to half of the 126 MB L2; beyond that the heads in flight at a time should be few (by
-// size, a batch of prefill chunks over 411 MB of keys and values took 2366 us instead of 2085, nine packed sequences with
-// 91 and 365 MB 2780 instead of 2730).  With that much work a launch has many rounds of blocks and its end matters little:
-// 1 % at 32768 tokens x 32 heads, whereas at 8192 x 16 the busiest SM had 1.54 times the mean of the backward's tiles and
-// 1.31 of the forward's, by size 1.13 and 1.04 (1385 us for both, by size 1165).
-inline int order_by_size(long long bytes, long long blocks) { return bytes <= (64ll << 20) && blocks < (1ll << 31); }
+// The rule.  By size where (figures: times in the order of the heads over times by size)
+// - what the blocks of different heads share only among themselves (`bytes`: K and V in the forward, Q and dO in the
+//   backward) is at most `most`.  Beyond that the heads in flight at a time should be few.  Forward, 72 MiB: 1.23 at 13 MB and
+//   1.02-1.07 at 62-74 MB; 82-93 MB 1.00-1.11 with up to 128 columns but 0.96 with 256; 98-143 MB 0.99-1.02 (256 columns, 164 MB: 0.88).
+//   Backward, 192 MiB: 1.05-1.38 at 40-186 MB (once 1.00), 1.08-1.16 at 197 MB, but 0.86-1.08 at 238-287 MB and 0.84-1.00
+//   beyond 350 MB.  The backward's bytes are streamed by many key blocks at once and need not stay.
+// - there are more blocks than SMs.  Otherwise all of them run at once and only lose their neighbours (backward, 128
+//   blocks: 0.96-0.99; 188-192: 0.98-1.19; 256: 1.06-1.30).
+// - a block's number says how long it is: its sequence has at most four times as many keys as queries (bound by the
+//   longest ones where each sequence has its own).  Behind a long prefix all blocks are about equally long, and those of one
+//   sequence belong together: paged chunks of 1024 behind 4000 keys 0.85-0.97, packed ones of 512 behind 6000 0.94-0.98, of
+//   1024 behind 2000-3000 1.01-1.09, of 2048 behind 500 1.13-1.35; 4096 x 16384 0.93 (gated) and 1.04 (dense).
+inline int order_by_size(long long bytes, long long most, long long blocks, int sms, int N, int Nk) {
+  return bytes <= most && blocks > sms && blocks < (1ll << 31) && Nk <= 4ll * N;
+}
 
 // ------------------------------------------------------------------------------------------------
 // programmatic dependent launch: a kernel lets its dependents be launched before it has finished; a dependent waits until
