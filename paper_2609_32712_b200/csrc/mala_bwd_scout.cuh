@@ -265,9 +265,8 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_con
         const int j = ja + kb, i = i0p + hf;
         const bool legal = i < T && i >= (kb ? i0b : i0a);     // (the other half of the pair / the first key block only)
         const bool valid_key = (j * 128 + rl) < Nkeys;
-        ok = mbar_wait(&s_full[buf], use & 1, status);
-        if (ok) ok = mbar_wait(&vec_full[buf], use & 1, status);
-        ok = __all_sync(0xffffffffu, ok);
+        ok = mbar_wait_warp(&s_full[buf], use & 1, status);
+        if (ok) ok = mbar_wait_warp(&vec_full[buf], use & 1, status);
         ++use;
         if (!ok) continue;
         tc_fence_after();

@@ -602,9 +602,8 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
 #pragma unroll
       for (int i = 0; i < NG; ++i) if (i == k) { ne = ne_k[i]; ++ne_k[i]; }
       const int ip = ne & 1;
-      ok = mbar_wait(&item_done[k][ip], (uint32_t)((ne >> 1) & 1), status);
-      ok = ok && mbar_wait(&st_full[k][ip], (uint32_t)((ne >> 1) & 1), status);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = mbar_wait_warp(&item_done[k][ip], (uint32_t)((ne >> 1) & 1), status);
+      ok = ok && mbar_wait_warp(&st_full[k][ip], (uint32_t)((ne >> 1) & 1), status);
       if (!ok) break;
       tc_fence_after();
       float ms[GH], ls[GH], ys[GH];
@@ -664,8 +663,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       if (publisher) { xch[k][half][xb][w][pub_row] = mx_w; xch[k][half][xb][w][8 + pub_row] = psum_w; }
       __syncwarp();
       if (lane == 0) mbar_arrive(&grp_bar[k][half]);
-      bool kk = mbar_wait(&grp_bar[k][half], xc & 1, status);
-      kk = __all_sync(0xffffffffu, kk);
+      const bool kk = mbar_wait_warp(&grp_bar[k][half], xc & 1, status);
       ++xc;
       if (!kk) return false;
       float a0[GS], a1[GS], a2[GS], a3[GS];
@@ -717,8 +715,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       for (int q = 0; q < (kLocalSums ? GS : 1); ++q) lacc[q] = 0.f;
       for (int t = 0; t < T; ++t, ++g) {
         const int sb = g & 3;
-        ok = mbar_wait(&s_full[k][sb], (uint32_t)((g >> 2) & 1), status);
-        ok = __all_sync(0xffffffffu, ok);
+        ok = mbar_wait_warp(&s_full[k][sb], (uint32_t)((g >> 2) & 1), status);
         if (!ok) break;
         tc_fence_after();
         // the leading parts and the remainders of this thread's heads
@@ -771,8 +768,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           mbar_arrive(&vote_bar[k][g & 3]);
         }
         if (!kDense && kSplit && !retain) {   // this half's heads would skip the tile: the other half's decide
-          ok = mbar_wait(&vote_bar[k][g & 3], (uint32_t)((g >> 2) & 1), status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = mbar_wait_warp(&vote_bar[k][g & 3], (uint32_t)((g >> 2) & 1), status);
           if (!ok) break;
           retain = (*(volatile int*)&flag[k][0][g & 7] | *(volatile int*)&flag[k][1][g & 7]) != 0;
           retain = __all_sync(0xffffffffu, retain);
@@ -806,8 +802,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             }
           }
           if (touch) {
-            ok = mbar_wait(&p_free[k][(rg - 1) % PP], (uint32_t)(((rg - 1) / PP) & 1), status);
-            ok = __all_sync(0xffffffffu, ok);
+            ok = mbar_wait_warp(&p_free[k][(rg - 1) % PP], (uint32_t)(((rg - 1) / PP) & 1), status);
             if (!ok) break;
             tc_fence_after();
             if constexpr (kSplit) {
@@ -838,8 +833,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           }
         }
         if (rg >= PP) {
-          ok = mbar_wait(&p_free[k][ps], (uint32_t)(((rg / PP) - 1) & 1), status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = mbar_wait_warp(&p_free[k][ps], (uint32_t)(((rg / PP) - 1) & 1), status);
           if (!ok) break;
         }
         float e[GS], pp[GS];

@@ -698,9 +698,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
 #pragma unroll
     for (int q = 0; q < GH; ++q) pend_l[q] = 1.f;
     auto flush = [&]() -> bool {
-      bool k = mbar_wait(&item_done[pend_ip], (uint32_t)((pend_ne >> 1) & 1), status);
-      k = __all_sync(0xffffffffu, k);
-      if (!k) return false;
+      if (!mbar_wait_warp(&item_done[pend_ip], (uint32_t)((pend_ne >> 1) & 1), status)) return false;
       tc_fence_after();
       uint32_t o[LDN], o2[D > 128 ? LDN : 1];
       tmem_ld_cols<LDN>(tmem_addr(tb, lane_base, DecCfg::kColO + (uint32_t)pend_ip * 16u + (uint32_t)rb), o);
@@ -766,8 +764,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
         if (publisher) { xch_max[xb][grp][w][pub_row] = mx_row; xch_sum[xb][grp][w][pub_row] = psum; }
         __syncwarp();
         if (lane == 0) mbar_arrive(&grp_a[grp]);
-        bool k = mbar_wait(&grp_a[grp], xc & 1, status);
-        k = __all_sync(0xffffffffu, k);
+        const bool k = mbar_wait_warp(&grp_a[grp], xc & 1, status);
         ++xc;
         if (!k) return false;
         float a0[GH], a1[GH], a2[GH], a3[GH];
@@ -790,8 +787,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
       for (int t = 0; t < T; ++t, ++g) {
         if (pend && t == 2) { ok = flush(); if (!ok) break; }
         const int sb = g & 3;
-        ok = mbar_wait(&s_full[sb], (uint32_t)((g >> 2) & 1), status);
-        ok = __all_sync(0xffffffffu, ok);
+        ok = mbar_wait_warp(&s_full[sb], (uint32_t)((g >> 2) & 1), status);
         if (!ok) break;
         tc_fence_after();
         uint32_t sr[LDN];
@@ -821,8 +817,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
           mbar_arrive(&vote_bar[g & 3]);
         }
         if (!kDense && NG > 1) {   // the tile is retained if a row of either group needs it
-          ok = mbar_wait(&vote_bar[g & 3], (uint32_t)((g >> 2) & 1), status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = mbar_wait_warp(&vote_bar[g & 3], (uint32_t)((g >> 2) & 1), status);
           if (!ok) break;
           retain = (*(volatile int*)&flag[0][g & 3] | *(volatile int*)&flag[1][g & 3]) != 0;
           retain = __all_sync(0xffffffffu, retain);
@@ -858,8 +853,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
           if (resc) {   // (the same decision in every thread: it only depends on exchanged values)
             // every PV so far has landed: the latest one (number rg - 1) releases its P^T slot last.  (A parity wait
             // must be neither ahead of nor two phases behind its barrier; per slot this one is exactly in step.)
-            ok = mbar_wait(&p_free[(rg - 1) & 3], (uint32_t)(((rg - 1) >> 2) & 1), status);
-            ok = __all_sync(0xffffffffu, ok);
+            ok = mbar_wait_warp(&p_free[(rg - 1) & 3], (uint32_t)(((rg - 1) >> 2) & 1), status);
             if (!ok) break;
             tc_fence_after();
             uint32_t o[LDN];
@@ -883,8 +877,7 @@ mala_decode_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
         // P^T into slot rg & 3 of its ring, free once the PV that last read it has retired
         const int ps = rg & 3;
         if (rg >= 4) {
-          ok = mbar_wait(&p_free[ps], (uint32_t)(((rg >> 2) - 1) & 1), status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = mbar_wait_warp(&p_free[ps], (uint32_t)(((rg >> 2) - 1) & 1), status);
           if (!ok) break;
         }
         {

@@ -423,8 +423,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
     for (int t = 0; t < T; ++t) {
       const int j = j0 - first - t;
-      ok = mbar_wait(&s_full[x], t & 1, status);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = mbar_wait_warp(&s_full[x], t & 1, status);
       if (!ok) break;
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
@@ -474,8 +473,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // A warp that found a retaining row knows the outcome (the vote is an OR) and goes straight on; only a warp
         // without one has to wait for the other three.
         if (!any) {
-          ok = mbar_wait(&vote_bar[x], t & 1, status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = mbar_wait_warp(&vote_bar[x], t & 1, status);
           if (!ok) break;
           retain = (*(volatile int*)&flag[x][t % 3]) != 0;
         }
@@ -485,8 +483,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (!kDense && hasB) {
           const int idx = (x == 0) ? t : (t - 1 - firstA);
           if (idx >= 0) {
-            ok = mbar_wait(&turn_bar[x], idx & 1, status);
-            ok = __all_sync(0xffffffffu, ok);
+            ok = mbar_wait_warp(&turn_bar[x], idx & 1, status);
             if (!ok) break;
           }
           __syncwarp();
@@ -538,9 +535,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // every waiter sees the phases in sequence.
       {
         const int idx = (x == 0) ? t : (t - 1 - firstA);
-        bool okw = true;
-        if (hasB && idx >= 0) okw = mbar_wait(&turn_bar[x], idx & 1, status);
-        ok = __all_sync(0xffffffffu, okw);
+        if (hasB && idx >= 0) ok = mbar_wait_warp(&turn_bar[x], idx & 1, status);
         if (!ok) break;
       }
       // P = exp2(s * c2 - m_ref), row sum in fp32 before the bf16 cast, P written over S
@@ -583,8 +578,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
     if (ok && present_x) {
       // finalize once every PV has retired: O <- O / l, lse <- m + log l
-      ok = mbar_wait(&fin_bar, 0, status);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = mbar_wait_warp(&fin_bar, 0, status);
     }
     if (ok && present_x && p.num_splits > 1) {
       // one range of the keys: normalised fp32 partial and the range's log-normalizer
