@@ -13,6 +13,7 @@
 #include "mala_bwd.cuh"
 #include "mala_decode.cuh"
 #include "mala_fwd.cuh"
+#include "mala_fwd_one.cuh"
 #include "tensor_map.h"
 
 namespace mala {
@@ -68,6 +69,13 @@ static bool set_smem(K kernel, int bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
 }
 
+template <int D>
+static bool set_smem_one() {
+  constexpr int bytes = FwdOneCfg<D>::kSmemBytes;
+  return set_smem(mala_fwd_one_kernel<D, true>, bytes) && set_smem(mala_fwd_one_kernel<D, false>, bytes) &&
+         set_smem(mala_fwd_one_kernel<D, true, true>, bytes) && set_smem(mala_fwd_one_kernel<D, false, true>, bytes);
+}
+
 // SMs of a device, asked for once.
 static int sm_count(int dev) {
   static std::atomic<int> known[64];
@@ -95,10 +103,7 @@ static int device_setup(int dev, int** status_out) {
     ok = ok && set_smem(mala_fwd_kernel<128, false, true>, FwdCfg<128, false>::kSmemBytes);
     ok = ok && set_smem(mala_fwd_kernel<64, false, true>, FwdCfg<64, false>::kSmemBytes);
     ok = ok && set_smem(mala_fwd_kernel<64, true, true>, FwdCfg<64, true>::kSmemBytes);
-    ok = ok && set_smem(mala_fwd_kernel<256, true>, FwdCfg<256, true>::kSmemBytes);
-    ok = ok && set_smem(mala_fwd_kernel<256, false>, FwdCfg<256, false>::kSmemBytes);
-    ok = ok && set_smem(mala_fwd_kernel<256, true, true>, FwdCfg<256, true>::kSmemBytes);
-    ok = ok && set_smem(mala_fwd_kernel<256, false, true>, FwdCfg<256, false>::kSmemBytes);
+    ok = ok && set_smem_one<64>() && set_smem_one<128>() && set_smem_one<256>();
     ok = ok && bwd_set_attributes();
     ok = ok && decode_set_attributes();
     if (!ok) return MALA_ERR_CUDA;
@@ -177,16 +182,26 @@ struct ApiScope {
 
 static const float kLog2e = 1.4426950408889634f;
 
-// Forward (prefill) launch: two query blocks per CTA (one with D = 256 or p.single).
-template <int D, bool kDense>
-static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& p,
-                      cudaStream_t stream) {
-  dim3 grid(FwdCfg<D, kDense>::kOne || p.single ? p.Tr : (p.Tr + 1) / 2, p.Hq, p.B * (p.num_splits > 1 ? p.num_splits : 1));
-  if (p.ppt > 1)
-    mala_fwd_kernel<D, kDense, true><<<grid, FwdCfg<D, kDense>::kThreads, FwdCfg<D, kDense>::kSmemBytes, stream>>>(tq, tk, tv, p);
-  else
-    mala_fwd_kernel<D, kDense><<<grid, FwdCfg<D, kDense>::kThreads, FwdCfg<D, kDense>::kSmemBytes, stream>>>(tq, tk, tv, p);
+// Forward (prefill) launch: two query blocks per CTA, or one (`one`; always above 128 columns).
+template <int D, bool kDense, bool kSmall>
+static int launch_fwd_as(bool one, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& p,
+                         cudaStream_t stream) {
+  dim3 grid(p.Tr, p.Hq, p.B * (p.num_splits > 1 ? p.num_splits : 1));
+  if constexpr (D <= 128) {
+    if (!one) {
+      grid.x = (p.Tr + 1) / 2;
+      mala_fwd_kernel<D, kDense, kSmall><<<grid, FwdCfg<D, kDense>::kThreads, FwdCfg<D, kDense>::kSmemBytes, stream>>>(tq, tk, tv, p);
+      return cudaGetLastError() == cudaSuccess ? MALA_OK : MALA_ERR_CUDA;
+    }
+  }
+  mala_fwd_one_kernel<D, kDense, kSmall><<<grid, FwdOneCfg<D>::kThreads, FwdOneCfg<D>::kSmemBytes, stream>>>(tq, tk, tv, p);
   return cudaGetLastError() == cudaSuccess ? MALA_OK : MALA_ERR_CUDA;
+}
+template <int D>
+static int launch_fwd(bool dense, bool one, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& p,
+                      cudaStream_t stream) {
+  if (p.ppt > 1) return dense ? launch_fwd_as<D, true, true>(one, tq, tk, tv, p, stream) : launch_fwd_as<D, false, true>(one, tq, tk, tv, p, stream);
+  return dense ? launch_fwd_as<D, true, false>(one, tq, tk, tv, p, stream) : launch_fwd_as<D, false, false>(one, tq, tk, tv, p, stream);
 }
 
 }  // namespace mala
@@ -360,16 +375,19 @@ static int fwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse,
   }
   p.scale_log2 = scale * kLog2e;
   p.log2_tau = tau > 0.f ? log2f(tau) : -INFINITY;
-  // Where every query block can have an SM of its own, it gets one: the call then takes as long as its longest block, and
-  // a block alone walks its tiles faster than two that share a CTA (1024 tokens, 2 heads of 64 columns: 17.3 us instead of
-  // 21.0; 512 tokens, 32 heads of 128: 14.1 instead of 17.5).
-  // Beyond that two blocks per CTA share the K tiles and hide one another's softmax.
-  p.single = (long long)p.Tr * Hq * B * num_splits <= sm_count(dev);
+  // One query block per CTA (mala_fwd_one.cuh) or two: the kernel for one walks a tile in 2100-2800 clk, the one for two takes
+  // 3800 for a tile of either.  So up to an SM per block a CTA has one: the call takes as long as its longest block (2048 tokens, 8
+  // heads of 128 columns 27 us, two blocks per CTA 44; 1024 tokens, 2 heads of 64: 16 and 23).  In causal self-attention, where the
+  // short blocks fill the SMs that the long ones leave, up to two blocks per SM (2048 tokens, 16 heads, 256 blocks: 31 and 45
+  // with 128 columns, 29 and 37 with 64; 24 heads, 384 blocks: 47 and 45, 43 and 38).  Beyond that two blocks per CTA share
+  // the K and V tiles and hide one another's softmax (8192 tokens, 16 heads of 128: 285 us, with one 317).
+  const long long all_blocks = (long long)p.Tr * Hq * B * num_splits;
+  const bool one = D == 256 || all_blocks <= (causal && Nk == N && !cu_k && !pg ? 2 : 1) * (long long)sm_count(dev);
   // (pages: at most the ones that the block tables can name, however large the pool is)
   const long long keys = pg ? (long long)(pg->num_pages < (long long)B * pg->max_pages_per_seq
                                               ? pg->num_pages : (long long)B * pg->max_pages_per_seq) * pg->page_size
                             : (long long)Bt * Nkt;
-  const long long blocks = (long long)(p.single || D == 256 ? p.Tr : (p.Tr + 1) / 2) * Hq * B * num_splits;
+  const long long blocks = (long long)(one ? p.Tr : (p.Tr + 1) / 2) * Hq * B * num_splits;
   p.by_size = order_by_size(4ll * d * Hkv * keys, 72ll << 20, blocks, sm_count(dev), N, Nk);
   if (p.bitmask) {
     if (cudaMemsetAsync(p.bitmask, 0, (size_t)B * Hq * p.Tr * p.words * sizeof(uint32_t), stream) != cudaSuccess)
@@ -380,9 +398,9 @@ static int fwd_impl(mala_tin q, mala_tin k, mala_tin v, mala_tout o, float* lse,
     return MALA_ERR_CUDA;
   const bool dense = (tau == 0.f);
   int rc;
-  if (D == 256) rc = dense ? launch_fwd<256, true>(tq, tk, tv, p, stream) : launch_fwd<256, false>(tq, tk, tv, p, stream);
-  else if (D == 128) rc = dense ? launch_fwd<128, true>(tq, tk, tv, p, stream) : launch_fwd<128, false>(tq, tk, tv, p, stream);
-  else rc = dense ? launch_fwd<64, true>(tq, tk, tv, p, stream) : launch_fwd<64, false>(tq, tk, tv, p, stream);
+  if (D == 256) rc = launch_fwd<256>(dense, one, tq, tk, tv, p, stream);
+  else if (D == 128) rc = launch_fwd<128>(dense, one, tq, tk, tv, p, stream);
+  else rc = launch_fwd<64>(dense, one, tq, tk, tv, p, stream);
   if (rc != MALA_OK || num_splits == 1) return rc;
   auto merge = D == 256 ? fwd_merge_splits_kernel<256> : D == 128 ? fwd_merge_splits_kernel<128> : fwd_merge_splits_kernel<64>;
   // (all rows in the grid's first coordinate: the others end at 65535, and B * Hq does not)

@@ -1,5 +1,5 @@
-// MALA forward (Algorithm 1) for sm_100a, prefill version: two query blocks per CTA (one with a head size above 128, and
-// where there is an SM for every query block).
+// MALA forward (Algorithm 1) for sm_100a, prefill version: two query blocks per CTA, head sizes up to 128 (mala_fwd_one.cuh:
+// one block per CTA, for larger heads and small calls).
 //
 // One CTA owns the two consecutive 128-row query blocks A = 2c and B = 2c+1 of one (batch, query
 // head).  They share the K tiles; each block has its own UMMA-issuing warp, softmax warpgroup,
@@ -59,7 +59,6 @@ struct FwdParams {
   // log-normalizer of the range; a merge kernel combines the ranges.
   int num_splits, tps;
   float* o_part;                 // [B, Hq, num_splits, N, D]
-  int single;                    // one query block per CTA instead of two
   int by_size;                   // see block_place
   int d;                         // head size of the tensors (<= D; the columns d .. D-1 are zeros and never stored)
   float* lse_part;               // [B, Hq, num_splits, N] natural log
@@ -71,12 +70,9 @@ template <int D, bool kDense>
 struct FwdCfg {
   static constexpr int kPanels = D / 64;
   static constexpr int kTileBytes = 128 * D * 2;
-  // Head sizes above 128: a tile is 64 KB, so a CTA owns ONE query block (block A; the warps of block B find no
-  // block) with one Q tile, one K stage and one V stage, and its accumulators S (128 columns) and O (256) fill the
-  // tensor memory that two blocks of 128 columns fill otherwise.
-  static constexpr bool kOne = D > 128;
-  static constexpr int kKStages = kOne ? 1 : 3;
-  static constexpr int kBlocks = kOne ? 1 : 2;     // Q tiles and V stages
+  static_assert(D <= 128, "two blocks of up to 128 columns fill the tensor memory");
+  static constexpr int kKStages = 3;
+  static constexpr int kBlocks = 2;                // Q tiles and V stages
   // Q_A, Q_B, K ring, V_A, V_B
   static constexpr int kSmemBytes = (kBlocks + kKStages + kBlocks) * kTileBytes + 1024;
   static constexpr int kThreads = 384;
@@ -91,7 +87,6 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                  const __grid_constant__ CUtensorMap tmV, const FwdParams p) {
   using Cfg = FwdCfg<D, kDense>;
   constexpr int KS = Cfg::kKStages, PAN = Cfg::kPanels, VS = Cfg::kBlocks;
-  constexpr bool kOne = Cfg::kOne;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sQ = smem;                               // [2] blocks A, B
@@ -144,13 +139,12 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int Tr = p.cu ? (Nq + qshift + 127) / 128 : p.Tr;
   const int Tk = p.cu ? (Nkeys + 127) / 128 : p.Tk;
   const int bz = p.cu ? 0 : b;                        // outermost TMA coordinate
-  const bool one = kOne || p.single;
-  const int npairs = one ? Tr : (Tr + 1) / 2;
+  const int npairs = (Tr + 1) / 2;
   // longest pairs first: of this head and sequence, or (by_size) of all of them, the longest sequence's last pair in front
   const int c = (p.by_size ? (int)gridDim.x : npairs) - 1 - place.x;
   if (c < 0 || c >= npairs) return;                  // (a sequence shorter than the longest one)
-  int iA = one ? c : 2 * c, iB = one ? c : 2 * c + 1;
-  bool hasB = !one && iB < Tr;
+  int iA = 2 * c, iB = 2 * c + 1;
+  bool hasB = iB < Tr;
   int dA = p.causal ? iA + koff : Tk - 1;            // newest key block with a legal key, per block
   const int dB = p.causal ? iB + koff : Tk - 1;
   int jlo = 0, jhi = Tk - 1;                         // key blocks of this CTA
@@ -412,7 +406,9 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const int first = (x == 0) ? firstA : 0;
     const int T = present_x ? (U - first) : 0;       // tiles of this block
     const bool mask_first = x ? (hB == dB) : (hA == dA);
-    float m_ref = -INFINITY, l = 0.f;
+    // (l: sum of the keys 0-63 of the tiles, and of the keys 64-127 -- in this order, because mala_fwd_one_kernel has a thread for
+    // either, and a row comes out the same bit for bit whichever kernel its call takes)
+    float m_ref = -INFINITY, l0 = 0.f, l1 = 0.f, l = 0.f, lg = -INFINITY;
     int r = 0;
     bool ok = true;
     uint32_t bm_bits = 0;
@@ -460,9 +456,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       bool retain = true;
       if (!kDense) {
         // Eq. 3: skip iff rowmax - (m + log l) < log(tau / L) for every valid row
-        bool vote;
-        if (l == 0.f) vote = valid;   // nothing retained yet: the log-ratio is +inf
-        else vote = valid && !(((mt - (m_ref + __log2f(l))) - theta) < 0.f);
+        const bool vote = valid && !((mt - lg) - theta < 0.f);   // (nothing retained yet: lg = -inf)
         const bool any = __any_sync(0xffffffffu, vote);
         if (lane == 0) {
           if (any) *(volatile int*)&flag[x][t % 3] = 1;
@@ -513,7 +507,8 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (need_any) {
           const float m_new = fmaxf(m_ref, mt);
           const float alpha = fast_exp2(m_ref - m_new);
-          l *= alpha;
+          l0 *= alpha;
+          l1 *= alpha;
           m_ref = m_new;
 #pragma unroll
           for (int cc = 0; cc < D / 32; ++cc) {
@@ -557,6 +552,8 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       }
       MALA_P_CHUNK(s0, 0)
       MALA_P_CHUNK(s1, 16)
+      l0 += (sum0 + sum1) + (sum2 + sum3);
+      sum0 = sum1 = sum2 = sum3 = 0.f;
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
@@ -568,7 +565,9 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (lane == 0 && hasB && (x == 0 || t >= firstA)) mbar_arrive(&turn_bar[1 - x]);
       MALA_P_CHUNK(s3, 48)
 #undef MALA_P_CHUNK
-      l += (sum0 + sum1) + (sum2 + sum3);
+      l1 += (sum0 + sum1) + (sum2 + sum3);
+      l = l0 + l1;
+      if (!kDense) lg = m_ref + __log2f(l);
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();

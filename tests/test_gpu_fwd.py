@@ -119,3 +119,23 @@ def test_fwd_near_threshold_decisions(mala, oracle, capsys):
         print(f"\n[near-threshold forward] tiles with |C| < 1e-2: {near}, inside the 1e-3 band: {band}, "
               f"decisions that differ from the oracle (all inside the band): {flips}")
     assert near >= 10 and band >= 1, "the workload must put tiles next to the threshold"
+
+
+# One query block per CTA (mala_fwd_one.cuh): score levels of the key blocks, newest first, in nats.  One to seven tiles; every
+# order of retained and skipped tiles that the V copies ahead of the vote can meet; maxima that move the reference of the
+# exponentials while the product before is still running.
+@pytest.mark.parametrize("levels", [[0], [0, 0], [0, -30], [0, -30, 0], [0, 0, -30, 0], [0, -30, -30, 0, 0], [0, -30, 0, -30, 0, -30, 0],
+                                    [0, 20, 40, 60], [0, 30, -30, 30, 60, 0, 62], [0, 0, 0, -30, -30, -30, -30]])
+@pytest.mark.parametrize("d,tau", [(64, 1e-3), (128, 1e-3), (128, 0.0), (192, 1e-3), (256, 1e-3), (256, 0.0)])
+def test_fwd_one_block_orders(mala, oracle, d, tau, levels):
+    N = 128 * len(levels) - 5
+    g = torch.Generator().manual_seed(d + len(levels))
+    q, k, v = (torch.randn((1, N, 2, d), generator=g) * s for s in (0.3, 0.3, 1.0))
+    scale = d ** -0.5
+    T = len(levels)
+    for x, level in enumerate(levels):
+        k[:, 128 * (T - 1 - x):128 * (T - x), :, 0] = level / (8 * scale)
+    q[..., 0] = 8.0
+    w = {"q": q.bfloat16(), "k": k.bfloat16(), "v": v.bfloat16(), "scale": scale}
+    r = _run_and_check(mala, oracle, w, tau, rounding_bound=True)
+    assert r["retained"] > 0 and (tau == 0.0 or r["skipped"] > 0 or min(levels) == 0)
