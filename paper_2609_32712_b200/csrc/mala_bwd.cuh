@@ -122,7 +122,7 @@ struct ListIter {
   }
 };
 
-constexpr int kBwdListWords = 4096;   // mask words of one CTA's G rows held in shared memory (list mode)
+constexpr int kBwdListWords = 2048;   // mask words of one CTA's G rows held in shared memory (list mode)
 
 // kList (with kDense): the tiles are those of the mask rows in p.list_mask, all of them retained: no test, no votes,
 // the dense tile pipeline on a sparse tile sequence.
@@ -884,8 +884,8 @@ inline bool bwd_set_attributes() {
   ok = ok && cudaFuncSetAttribute(mala_bwd_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<64>::kSmemBytes) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(mala_bwd_kernel<128, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<128>::kSmemBytes) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(mala_bwd_kernel<64, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<64>::kSmemBytes) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(mala_bwd_scout_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoutCfg<128>::kSmemBytes) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(mala_bwd_scout_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoutCfg<64>::kSmemBytes) == cudaSuccess;
+  ok = ok && cudaFuncSetAttribute(mala_bwd_scout_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoutCfg<128>::kMaxSmem) == cudaSuccess;
+  ok = ok && cudaFuncSetAttribute(mala_bwd_scout_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoutCfg<64>::kMaxSmem) == cudaSuccess;
   return ok;
 }
 
@@ -897,10 +897,14 @@ inline int bwd_launch_main(const CUtensorMap& tq, const CUtensorMap& tk, const C
   return cudaGetLastError() == cudaSuccess ? MALA_OK : MALA_ERR_CUDA;
 }
 
+// Four key blocks per CTA, or two where four would give the SMs less than two CTAs each; as many Q tiles in the ring as the masks
+// leave room for.
 template <int D>
-inline int bwd_launch_scout(const CUtensorMap& tq, const CUtensorMap& tk, const ScoutParams& sp, cudaStream_t stream) {
-  dim3 grid((sp.Tk + 1) / 2, sp.Hkv, sp.B);
-  mala_bwd_scout_kernel<D><<<grid, ScoutCfg<D>::kThreads, ScoutCfg<D>::kSmemBytes, stream>>>(tq, tk, sp);
+inline int bwd_launch_scout(const CUtensorMap& tq, const CUtensorMap& tk, ScoutParams& sp, int sms, cudaStream_t stream) {
+  sp.pairs = (long long)((sp.Tk + 3) / 4) * sp.Hq * sp.B >= 2ll * sms ? 2 : 1;
+  sp.stages = ScoutCfg<D>::bytes(sp.pairs, 3, sp.wpad) <= ScoutCfg<D>::kMaxSmem ? 3 : 2;
+  dim3 grid((sp.Tk + 2 * sp.pairs - 1) / (2 * sp.pairs), sp.Hq, sp.B);
+  mala_bwd_scout_kernel<D><<<grid, ScoutCfg<D>::kThreads, ScoutCfg<D>::bytes(sp.pairs, sp.stages, sp.wpad), stream>>>(tq, tk, sp);
   return cudaGetLastError() == cudaSuccess ? MALA_OK : MALA_ERR_CUDA;
 }
 
@@ -971,7 +975,7 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
   // (whole backward, 1024 tokens, 2 heads of 64 columns: 27.7 us instead of 39.8, 29.9 instead of 42.2 with 128 columns and
   // nearly every tile skipped; 512 tokens, 32 / 8 heads: 61 instead of 87).
   const bool brief = (long long)Tk * Hkv * B <= sms && (Hq / Hkv) * T <= 16;
-  const bool two_pass = !dense && !brief && MALA_BWD_TWO_PASS && (Hq / Hkv) * 2 * wpad <= kScoutMaskWords && (Hq / Hkv) <= 16 &&
+  const bool two_pass = !dense && !brief && MALA_BWD_TWO_PASS && (Hq / Hkv) * wpad <= kBwdListWords && (Hq / Hkv) <= 16 &&
                         ws_bytes >= base_bytes + bwd_list_bytes(B, Hq, T, Tk);
   int rc;
   if (two_pass) {
@@ -987,9 +991,7 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
     sp.scale_log2 = p.scale_log2;
     sp.sample = MALA_BWD_SAMPLE;
     sp.by_size = p.by_size;
-    CUtensorMap tq2;   // the queries again, in boxes of two tiles
-    if (!make_tensor_map_bnhd(&tq2, q.p, Bl, Nt, Hq, d, q.sb, q.sn, q.sh, 256)) return MALA_ERR_TENSOR_MAP;
-    rc = (D == 128) ? bwd_launch_scout<128>(tq2, tk, sp, stream) : bwd_launch_scout<64>(tq2, tk, sp, stream);
+    rc = (D == 128) ? bwd_launch_scout<128>(tq, tk, sp, sms, stream) : bwd_launch_scout<64>(tq, tk, sp, sms, stream);
     if (rc != MALA_OK) return rc;
     BwdParams pl = p;
     pl.retained = nullptr; pl.bitmask = nullptr; pl.totals = nullptr;   // (the first pass wrote the telemetry of these rows)

@@ -2,29 +2,31 @@
 //
 // The backward test of a tile depends only on its scores and on the saved log-normalizers, not on any other tile, so
 // the retained support of a key block can be found before any gradient work starts.  This kernel does that at the rate
-// the tensor pipe forms the scores: one CTA per (pair of key blocks, KV head, batch) keeps both K tiles in shared
-// memory and streams the Q tiles of the group's query heads, two at a time, through a ring of two 256-row stages; a
-// pair of Q tiles feeds two MMA batches S^T = K_j [Q_i; Q_i+1]^T of shape 128 x 256, one per key block, into two TMEM
-// buffers of 256 columns, and four warpgroups -- one per 128-column half of a buffer -- read and test their score tile
-// while the other buffer is being formed.  (Why this shape: with one key block per CTA the kernel was bound by the
-// delivery of the Q tiles, 32 KB per score tile from L2; with 128 x 128 MMAs it was bound by shared-memory bandwidth,
-// which an SS MMA of that shape takes whole, leaving none for the copies that refill the ring; a 128 x 256 MMA reads
-// 12 KB per 128 clk and leaves a quarter of it.)  Nothing waits for a vote: a warp that finds a retained entry sets the tile's bit in a shared-memory copy of
+// the tensor pipe forms the scores.  One CTA per (two or four key blocks, query head, batch) keeps the K tiles in shared memory
+// and streams the head's Q tiles through a ring; a Q tile and a pair of key blocks make one MMA batch S = Q_i [K_j; K_j+1]^T of
+// shape 128 x 256 into one of two TMEM buffers of 256 columns, and four warpgroups -- one per key block of a buffer -- read and
+// test their score tile while the other buffer is being formed.  The queries are the rows: a thread owns one, and the test of its
+// 128 scores is one comparison of their largest (max_e (s_e c2) >= bq <=> some s_e c2 >= bq; fma is monotone).
+//
+// Bound by the tensor pipe: 512 clk per tile.  Why this shape: a 128 x 128 MMA takes the whole bandwidth of shared memory and
+// leaves none for the copies that refill the ring, a 128 x 256 MMA three quarters; a Q tile serves four score tiles, with 16 bytes of
+// copies per clk and SM.  (With the keys as rows and pairs of Q tiles as columns it serves two, and every column has a threshold of
+// its own: 8192 tokens, 16 / 4 heads of 128 columns, a third of the tiles retained: 157 us, now 98; 131072 tokens, 8 / 2 heads: 9.4
+// and 8.9 ms, where the 1.55 PFLOP/s of tested tiles are what the power limit allows.)
+// Nothing waits for a vote: a warp that finds a retained entry sets the tile's bit in a shared-memory copy of
 // the row's mask, and the row is written out when the head's last tile has been tested.  The second pass
 // (mala_bwd_kernel in its list mode) then visits the retained tiles only and runs the dense tile pipeline on them.
 //
 // Rows that retain everything gain nothing from a first pass (their scores would be formed twice), so the rows of a
-// CTA are sampled first: every eighth tile of every head.  A head whose sampled tiles are all retained, for both key
-// blocks of the pair, is left to the one-pass kernel (mala_bwd_kernel without the list, restricted to such heads), which
-// tests and works tile by tile; only the other heads are tested in full here.
+// CTA are sampled first: two tiles of every sixteen.  If all of them are retained, for every key block of the CTA, the head's rows
+// are left to the one-pass kernel (mala_bwd_kernel without the list, restricted to such heads), which tests and works tile by tile.
 //
 // Output, per (batch, query head, key block j): the row's mask (bit i set iff tile (j, i) is retained; rows padded to
 // a multiple of four words) and its number of set bits, or an empty mask and the count kScoutDirectRow for a row that
 // is left to the one-pass kernel.
 //
-// Warp roles (640 threads): warp 0 TMA producer (K_j once, Q ring), warp 1 UMMA issuer, warp 2 per-query test offsets
-// (bq = lse2 + log2(tau / L_q) of the tile's 128 queries into a ring of four shared-memory slots, with the minimum of
-// each 32-column chunk), warps 4-19 the four test groups (thread = key row).
+// Warp roles (640 threads): warp 0 TMA producer (K once, Q ring), warp 1 UMMA issuer, warps 2-3 idle, warps 4-19 the four test
+// groups (thread = query row).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -35,8 +37,7 @@
 namespace mala {
 
 constexpr uint32_t kScoutDirectRow = 0xffffffffu;   // row_count of a row left to the one-pass kernel
-constexpr int kScoutMaskWords = 4096;               // mask words of one CTA (G heads x 2 key blocks x wpad) in shared memory
-constexpr int kScoutSampleStride = 16;              // one pair of every sixteen tiles of a row is sampled first ...
+constexpr int kScoutSampleStride = 16;              // two tiles of every sixteen of a row are sampled first ...
 constexpr int kScoutSampleMinTiles = 32;            // ... in rows of at least this many tiles
 
 struct ScoutParams {
@@ -54,63 +55,60 @@ struct ScoutParams {
   int sample;                 // sample the rows first and leave the ones that retain everything to the one-pass kernel
   float scale_log2;
   int by_size;                // see block_place
+  int pairs, stages;          // key blocks of a CTA / 2 (1 or 2); Q tiles in the ring (2 or 3)
 };
 
 template <int D>
 struct ScoutCfg {
   static constexpr int kPanels = D / 64;
   static constexpr int kTileBytes = 128 * D * 2;
-  static constexpr int kPairBytes = 2 * kTileBytes;                      // two Q tiles: panels of 256 rows
-  static constexpr int kSmemBytes = 2 * kTileBytes + 2 * kPairBytes + 1024;   // K of two key blocks, ring of two Q pairs
+  static constexpr int kPairBytes = 2 * kTileBytes;                      // two K tiles: panels of 256 rows
   static constexpr int kThreads = 640;
+  static constexpr int kMaxSmem = 232448 - 1024;                         // (static: the barriers, rounded up)
+  static constexpr int bytes(int pairs, int stages, int wpad) {
+    return pairs * kPairBytes + stages * kTileBytes + 2 * pairs * wpad * 4 + 1024;
+  }
 };
 
-// The sequence of Q-tile pairs of a CTA, the same for every role: the sampled pairs of all heads, then -- once the
-// sampled votes have decided which heads are left to the one-pass kernel (`sync` returns after dflag[] has been
-// written) -- the other pairs of the other heads.  body(h, i) handles the Q tiles i, i + 1 of head h (i + 1 may lie
-// beyond the last tile); both return false to stop.
+// The sequence of Q tiles of a CTA, the same for every role: the sampled ones, then -- unless the sampled votes have left the
+// head to the one-pass kernel (`sync` returns after *direct has been written) -- the others.  body(i) returns false to stop.
 template <class Body, class Sync>
-__device__ __forceinline__ bool scout_for_each_pair(int G, int i0a, int T, bool sampling, const volatile int* dflag,
-                                                    Body body, Sync sync) {
+__device__ __forceinline__ bool scout_for_each_tile(int i0, int T, bool sampling, const volatile int* direct, Body body, Sync sync) {
   if (sampling) {
-    for (int h = 0; h < G; ++h)
-      for (int i = i0a; i < T; i += kScoutSampleStride)
-        if (!body(h, i)) return false;
+    for (int i = i0; i < T; i += ((i - i0) % kScoutSampleStride == 0) ? 1 : kScoutSampleStride - 1)
+      if (!body(i)) return false;
     if (!sync()) return false;
+    if (*direct) return true;
   }
-  for (int h = 0; h < G; ++h) {
-    if (sampling && dflag[h]) continue;
-    for (int i = i0a; i < T; i += 2) {
-      if (sampling && ((i - i0a) % kScoutSampleStride) == 0) continue;
-      if (!body(h, i)) return false;
-    }
+  for (int i = i0; i < T; ++i) {
+    if (sampling && ((i - i0) % kScoutSampleStride) < 2) continue;
+    if (!body(i)) return false;
   }
   return true;
 }
 
 template <int D>
 __global__ void __launch_bounds__(640, 1)
-mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_constant__ CUtensorMap tmK,
+mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const ScoutParams p) {
   using Cfg = ScoutCfg<D>;
   constexpr int PAN = Cfg::kPanels;
+  const int KB = 2 * p.pairs, QS = p.stages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sK = smem;                          // key blocks ja, jb
-  uint8_t* sQ = sK + 2 * Cfg::kTileBytes;      // 2 stages of two Q tiles each ([panel][256 rows][128 B])
+  uint8_t* sK = smem;                               // [pair][panel][256 rows][128 B]
+  uint8_t* sQ = sK + p.pairs * Cfg::kPairBytes;     // Q ring
+  uint32_t* rowmask = (uint32_t*)(sQ + QS * Cfg::kTileBytes);   // [key block][wpad]
 
-  __shared__ uint64_t k_full, q_full[2], q_empty[2], s_full[2], s_empty[2], vec_full[2], vec_empty[2], fin_bar, phase_bar;
-  __shared__ __align__(16) float vec[2][256];  // [batch & 1][query column of the pair]: bq
-  __shared__ float vmin[2][8];                 // [batch & 1][32-column chunk]: smallest bq of the chunk
-  __shared__ uint32_t rowmask[kScoutMaskWords];   // [head][key block of the pair][wpad]
-  __shared__ int dflag[16];                    // head is left to the one-pass kernel
+  __shared__ uint64_t k_full, q_full[3], q_empty[3], s_full[2], s_empty[2], fin_bar, phase_bar;
+  __shared__ int direct_s;                          // the head is left to the one-pass kernel
   __shared__ uint32_t tmem_base_s;
   __shared__ int early_exit;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const BlockPlace place = block_place(p.by_size);
-  const int ja = 2 * place.x, jb = ja + 1, hkv = place.y, b = place.z;
-  const int G = p.Hq / p.Hkv;
+  const int ja = KB * place.x, h = place.y, b = place.z;
+  const int hkv = h / (p.Hq / p.Hkv);
   // this sequence (the geometry of mala_bwd_kernel)
   const int row0 = p.cu ? __ldg(p.cu + b) : 0;
   const int Nq = p.cu ? __ldg(p.cu + b + 1) - row0 : p.N;
@@ -123,24 +121,21 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_con
   const int prow0 = p.cu ? ((row0 + (p.cu_k ? 384 : 128) * b) / 128) * 128 : 0;
   const int Tk_seq = p.cu ? (Nkeys + 127) / 128 : p.Tk;                      // key blocks of this sequence
   const bool none = p.cu_k && (Nq <= 0 || (p.causal && Nkeys < Nq));         // (no defined tile at all)
-  const bool has_a = !none && ja < Tk_seq, has_b = !none && jb < Tk_seq;
-  // Q tiles i0a .. T-1 of every head; the second key block's tile exists from i0b on
-  const int i0a = p.causal ? max(ja - koff, 0) : 0;
-  const int i0b = has_b ? (p.causal ? max(jb - koff, 0) : 0) : T;
-  const int ni = has_a ? T - i0a : 0;
+  const int nkb = none ? 0 : min(KB, Tk_seq - ja);                           // key blocks of this CTA (<= 0: none)
+  // tile (i, j) is legal from i = first(j) on
+  auto first = [&](int j) -> int { return p.causal ? max(j - koff, 0) : 0; };
+  const int i0 = first(ja);
+  const int ni = nkb > 0 ? T - i0 : 0;
   const bool sampling = p.sample && ni >= kScoutSampleMinTiles;
-  const size_t out_row0 = ((size_t)b * p.Hq + (size_t)hkv * G) * p.Tk;        // + h * Tk + j
+  const size_t out_row = ((size_t)b * p.Hq + h) * p.Tk + ja;
   const int wpad = p.wpad;
   int* status = p.status;
   if (ni <= 0) {   // key blocks without queries: empty rows
-    for (int kb = 0; kb < 2; ++kb) {
-      const int j = ja + kb;
-      if (j >= p.Tk) continue;
-      for (int x = tid; x < G * wpad; x += blockDim.x)
-        p.mask[(out_row0 + (size_t)(x / wpad) * p.Tk + j) * wpad + x % wpad] = 0u;
-      if (tid < G) {
-        p.row_count[out_row0 + (size_t)tid * p.Tk + j] = 0u;
-        if (p.tel_retained) p.tel_retained[out_row0 + (size_t)tid * p.Tk + j] = 0u;
+    for (int kb = 0; kb < KB && ja + kb < p.Tk; ++kb) {
+      for (int x = tid; x < wpad; x += blockDim.x) p.mask[(out_row + kb) * wpad + x] = 0u;
+      if (tid == 0) {
+        p.row_count[out_row + kb] = 0u;
+        if (p.tel_retained) p.tel_retained[out_row + kb] = 0u;
       }
     }
     return;
@@ -148,16 +143,14 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_con
 
   if (tid == 0) {
     early_exit = (*(volatile int*)status != 0);
+    direct_s = 0;
     mbar_init(&k_full, 1);
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&q_full[s], 1); mbar_init(&q_empty[s], 1); mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 8);
-      mbar_init(&vec_full[s], 1); mbar_init(&vec_empty[s], 8);
-    }
+    for (int s = 0; s < 3; ++s) { mbar_init(&q_full[s], 1); mbar_init(&q_empty[s], 1); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 8); }
     mbar_init(&fin_bar, 1); mbar_init(&phase_bar, 1);
     mbar_fence_init();
   }
-  for (int x = tid; x < G * 2 * wpad; x += blockDim.x) rowmask[x] = 0u;
-  if (tid < 16) dflag[tid] = 0;
+  for (int x = tid; x < KB * wpad; x += blockDim.x) rowmask[x] = 0u;
   __syncthreads();
   if (early_exit) return;
   if (warp == 0) { tmem_alloc(&tmem_base_s, 512); tmem_relinquish(); }
@@ -165,27 +158,25 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tb = tmem_base_s;
-  // An MMA batch per key block of the pair and Q pair: batch A always, batch B where the second key block has a legal
-  // tile in the pair.  Batch m goes to TMEM buffer m & 1.
-  auto batches = [&](int i) -> int { return (has_b && i + 1 >= i0b) ? 2 : 1; };
+  // An MMA batch per pair of key blocks and Q tile, where the pair has a legal tile.  Batch m goes to TMEM buffer m & 1.
+  auto batches = [&](int i) -> int { return (nkb > 2 && i >= first(ja + 2)) ? 2 : 1; };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&tmQ2); tma_prefetch_desc(&tmK);
-      mbar_arrive_expect_tx(&k_full, (has_b ? 2 : 1) * Cfg::kTileBytes);
-      for (int pn = 0; pn < PAN; ++pn) {
-        tma_load_4d(sK + pn * 16384, &tmK, &k_full, pn * 64, krow0 + ja * 128, hkv, bz);
-        if (has_b) tma_load_4d(sK + Cfg::kTileBytes + pn * 16384, &tmK, &k_full, pn * 64, krow0 + jb * 128, hkv, bz);
-      }
-      int n = 0;
-      scout_for_each_pair(G, i0a, T, sampling, dflag, [&](int h, int i) -> bool {
-        const int s = n & 1;
-        if (!mbar_wait(&q_empty[s], ((n >> 1) & 1) ^ 1, status)) return false;
-        mbar_arrive_expect_tx(&q_full[s], Cfg::kPairBytes);
-        for (int pn = 0; pn < PAN; ++pn)   // (rows past the tensor read as zeros; a second tile past the head's last one is ignored)
-          tma_load_4d(sQ + s * Cfg::kPairBytes + pn * 32768, &tmQ2, &q_full[s], pn * 64, row0 + i * 128 - qshift, hkv * G + h, bz);
-        ++n;
+      tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK);
+      mbar_arrive_expect_tx(&k_full, nkb * Cfg::kTileBytes);
+      for (int kb = 0; kb < nkb; ++kb)
+        for (int pn = 0; pn < PAN; ++pn)
+          tma_load_4d(sK + (kb >> 1) * Cfg::kPairBytes + pn * 32768 + (kb & 1) * 16384, &tmK, &k_full, pn * 64, krow0 + (ja + kb) * 128, hkv, bz);
+      int s = 0;
+      uint32_t par = 1;
+      scout_for_each_tile(i0, T, sampling, &direct_s, [&](int i) -> bool {
+        if (!mbar_wait(&q_empty[s], par, status)) return false;
+        mbar_arrive_expect_tx(&q_full[s], Cfg::kTileBytes);
+        for (int pn = 0; pn < PAN; ++pn)   // (rows before and past the tensor read as zeros)
+          tma_load_4d(sQ + s * Cfg::kTileBytes + pn * 16384, &tmQ, &q_full[s], pn * 64, row0 + i * 128 - qshift, h, bz);
+        if (++s == QS) { s = 0; par ^= 1; }
         return true;
       }, [&]() -> bool { return mbar_wait(&phase_bar, 0, status); });
     }
@@ -193,170 +184,135 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ2, const __grid_con
     // ------------------------------------------------------------------ UMMA issuer (warp-uniform issue loop)
     const uint32_t leader = elect_one();
     constexpr uint32_t idesc = make_idesc_bf16(128, 256, false, false);
-    const uint64_t dKa = make_smem_desc(smem_u32(sK), 16, 1024);
-    const uint64_t dKb = make_smem_desc(smem_u32(sK + Cfg::kTileBytes), 16, 1024);
+    const uint64_t dK0 = make_smem_desc(smem_u32(sK), 16, 1024);
     const uint64_t dQ0 = make_smem_desc(smem_u32(sQ), 16, 1024);
     bool ok = mbar_wait_warp(&k_full, 0, status);
-    int n = 0, m = 0;
-    if (ok) scout_for_each_pair(G, i0a, T, sampling, dflag, [&](int h, int i) -> bool {
-      const int s = n & 1;
-      if (!mbar_wait_warp(&q_full[s], (n >> 1) & 1, status)) return false;
-      const uint64_t dQ = desc_advance(dQ0, s * Cfg::kPairBytes);
+    int s = 0, m = 0;
+    uint32_t par = 0;
+    if (ok) scout_for_each_tile(i0, T, sampling, &direct_s, [&](int i) -> bool {
+      if (!mbar_wait_warp(&q_full[s], par, status)) return false;
+      const uint64_t dQ = desc_advance(dQ0, s * Cfg::kTileBytes);
       const int nb = batches(i);
-      for (int kb = 0; kb < nb; ++kb, ++m) {
+      for (int pr = 0; pr < nb; ++pr, ++m) {
         const int buf = m & 1;
         if (!mbar_wait_warp(&s_empty[buf], ((m >> 1) & 1) ^ 1, status)) return false;   // the buffer's previous batch has been read
         tc_fence_after();
-        const uint64_t dK = kb ? dKb : dKa;
+        const uint64_t dK = desc_advance(dK0, pr * Cfg::kPairBytes);
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
-          mma_ss(tmem_addr(tb, 0, buf * 256), desc_advance(dK, (k >> 2) * 16384 + (k & 3) * 32),
-                 desc_advance(dQ, (k >> 2) * 32768 + (k & 3) * 32), idesc, k > 0, leader);
+          mma_ss(tmem_addr(tb, 0, buf * 256), desc_advance(dQ, (k >> 2) * 16384 + (k & 3) * 32),
+                 desc_advance(dK, (k >> 2) * 32768 + (k & 3) * 32), idesc, k > 0, leader);
         if (leader) tc_commit(&s_full[buf]);
       }
       if (leader) tc_commit(&q_empty[s]);
-      ++n;
+      if (++s == QS) { s = 0; par ^= 1; }
       return true;
     }, [&]() -> bool { return mbar_wait_warp(&phase_bar, 0, status); });
     __syncwarp();
     if (leader) tc_commit(&fin_bar);
     mbar_wait_warp(&fin_bar, 0, status);
-  } else if (warp == 2) {
-    // ------------------------------------------------------------------ test offsets of every batch's 256 queries
-    int m = 0;
-    scout_for_each_pair(G, i0a, T, sampling, dflag, [&](int h, int i) -> bool {
-      // lane l carries queries 8 l .. 8 l + 7 of the pair (a second tile past the head's last one reads what follows
-      // in the padded vector or +inf beyond it: never used)
-      const size_t x = ((size_t)bz * p.Hq + hkv * G + h) * p.Np + (size_t)prow0 + (size_t)i * 128 + lane * 8;
-      const bool in = (i + 1 < T) || lane < 16;
-      const float4 inf4 = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-      const float4 v0 = in ? *reinterpret_cast<const float4*>(p.bq + x) : inf4;
-      const float4 v1 = in ? *reinterpret_cast<const float4*>(p.bq + x + 4) : inf4;
-      float mn = fminf(fminf(fminf(v0.x, v0.y), fminf(v0.z, v0.w)), fminf(fminf(v1.x, v1.y), fminf(v1.z, v1.w)));
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
-      const int nb = batches(i);
-      for (int kb = 0; kb < nb; ++kb, ++m) {   // (one slot per batch: both key blocks get their copy)
-        const int s = m & 1;
-        if (!mbar_wait_warp(&vec_empty[s], ((m >> 1) & 1) ^ 1, status)) return false;
-        *reinterpret_cast<float4*>(&vec[s][lane * 8]) = v0;
-        *reinterpret_cast<float4*>(&vec[s][lane * 8 + 4]) = v1;
-        if ((lane & 3) == 0) vmin[s][lane >> 2] = mn;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&vec_full[s]);
-      }
-      return true;
-    }, [&]() -> bool { return mbar_wait_warp(&phase_bar, 0, status); });
   } else if (warp >= 4) {
-    // ------------------------------------------------------------------ test groups: group g takes the 128-column half g & 1
-    // (the Q tile i + (g & 1) of the pair) of the batches in buffer g >> 1
+    // ------------------------------------------------------------------ test groups: group g takes the key block g & 1 of the
+    // pair of the batches in buffer g >> 1
     const int g = (warp - 4) >> 2, buf = g >> 1, hf = g & 1;
     const uint32_t lane_base = (uint32_t)(warp & 3) * 32u;
     const int rl = (int)lane_base + lane;
     const float c2 = p.scale_log2;
     const int st = tid - 128;                      // 0 .. 511 among the test threads
+    const float* bq = p.bq + ((size_t)bz * p.Hq + h) * p.Np + (size_t)prow0 + rl;
     bool ok = true;                                // (a warp whose wait failed goes on through the barriers below)
     int use = 0;                                   // batches this group's buffer has held (parity of its barriers)
     int m = 0;
-    scout_for_each_pair(G, i0a, T, sampling, dflag, [&](int h, int i0p) -> bool {
-      const int nb = batches(i0p);
-      for (int kb = 0; kb < nb; ++kb, ++m) {
+    scout_for_each_tile(i0, T, sampling, &direct_s, [&](int i) -> bool {
+      const int nb = batches(i);
+      for (int pr = 0; pr < nb; ++pr, ++m) {
         if ((m & 1) != buf || !ok) continue;
-        const int j = ja + kb, i = i0p + hf;
-        const bool legal = i < T && i >= (kb ? i0b : i0a);     // (the other half of the pair / the first key block only)
-        const bool valid_key = (j * 128 + rl) < Nkeys;
+        const int kb = 2 * pr + hf, j = ja + kb;
+        const bool legal = kb < nkb && i >= first(j);
+        const float need = legal ? __ldg(bq + (size_t)i * 128) : INFINITY;   // (in flight while the scores are waited for)
         ok = mbar_wait_warp(&s_full[buf], use & 1, status);
-        if (ok) ok = mbar_wait_warp(&vec_full[buf], use & 1, status);
         ++use;
         if (!ok) continue;
         tc_fence_after();
-        const bool diag = p.causal && (i + koff == j);
         bool vote = false;
         if (legal) {
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t sc[32];
-            tmem_ld_x32(tmem_addr(tb, lane_base, buf * 256 + hf * 128 + c * 32), sc);
+          // keys that this row may see: up to its own on the diagonal tile, up to the last one in the ragged last block
+          int lim = min(128, Nkeys - j * 128);
+          if (p.causal && i + koff == j) lim = min(lim, rl + 1);
+          const bool cut = __any_sync(0xffffffffu, lim < 128);
+          float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            uint32_t sa[32], sb[32];
+            tmem_ld_x32(tmem_addr(tb, lane_base, buf * 256 + hf * 128 + c * 64), sa);
+            tmem_ld_x32(tmem_addr(tb, lane_base, buf * 256 + hf * 128 + c * 64 + 32), sb);
             tmem_wait_ld();
-            if (diag) {   // entry (key rl, query col) is legal iff rl <= col
+            if (cut) {
               const uint32_t ninf = 0xff800000u;
 #pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (c * 32 + e < rl) sc[e] = ninf;
-            }
-            // bound first: max_e (s_e c2 - bq_e) <= (max_e s_e) c2 - min_e bq_e (c2 > 0; fma is monotone in each argument)
-            float m0 = __uint_as_float(sc[0]), m1 = __uint_as_float(sc[1]);
-#pragma unroll
-            for (int e = 0; e < 7; ++e) {
-              m0 = max3(m0, __uint_as_float(sc[2 + 4 * e]), __uint_as_float(sc[3 + 4 * e]));
-              m1 = max3(m1, __uint_as_float(sc[4 + 4 * e]), __uint_as_float(sc[5 + 4 * e]));
-            }
-            const float mx = max3(m0, m1, fmaxf(__uint_as_float(sc[30]), __uint_as_float(sc[31])));
-            const bool cand = valid_key && !(fmaf(mx, c2, -vmin[buf][hf * 4 + c]) < 0.f);
-            if (__any_sync(0xffffffffu, cand)) {
-              const float4* bb = reinterpret_cast<const float4*>(vec[buf] + hf * 128) + c * 8;
-              float c0 = -INFINITY, c1 = -INFINITY;
-#pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                const float4 x0 = bb[e];
-                c0 = max3(c0, fmaf(__uint_as_float(sc[4 * e + 0]), c2, -x0.x), fmaf(__uint_as_float(sc[4 * e + 1]), c2, -x0.y));
-                c1 = max3(c1, fmaf(__uint_as_float(sc[4 * e + 2]), c2, -x0.z), fmaf(__uint_as_float(sc[4 * e + 3]), c2, -x0.w));
+              for (int e = 0; e < 32; ++e) {
+                if (c * 64 + e >= lim) sa[e] = ninf;
+                if (c * 64 + 32 + e >= lim) sb[e] = ninf;
               }
-              vote = vote || (valid_key && !(fmaxf(c0, c1) < 0.f));
             }
-            // (one retaining entry decides the tile: the other chunks need not be read)
-            if (__any_sync(0xffffffffu, vote)) break;
+#pragma unroll
+            for (int e = 0; e < 32; e += 4) {
+              m0 = max3(m0, __uint_as_float(sa[e]), __uint_as_float(sa[e + 1]));
+              m1 = max3(m1, __uint_as_float(sb[e]), __uint_as_float(sb[e + 1]));
+              m2 = max3(m2, __uint_as_float(sa[e + 2]), __uint_as_float(sa[e + 3]));
+              m3 = max3(m3, __uint_as_float(sb[e + 2]), __uint_as_float(sb[e + 3]));
+            }
           }
+          vote = fmaf(fmaxf(max3(m0, m1, m2), m3), c2, -need) >= 0.f;   // Eq. 4 (padding rows: need = +inf)
         }
-        tc_fence_before();
-        __syncwarp();
+        const bool any = __any_sync(0xffffffffu, vote);
         if (lane == 0) {
+          tc_fence_before();
           mbar_arrive(&s_empty[buf]);
-          mbar_arrive(&vec_empty[buf]);
+          if (any) atomicOr(&rowmask[kb * wpad + (i >> 5)], 1u << (i & 31));
         }
-        if (__any_sync(0xffffffffu, vote) && lane == 0) atomicOr(&rowmask[(h * 2 + kb) * wpad + (i >> 5)], 1u << (i & 31));
       }
       return true;
     }, [&]() -> bool {
-      // all sampled tiles have been tested once the sixteen warps meet here: a head whose samples are all retained,
-      // for both key blocks, is left to the one-pass kernel
+      // all sampled tiles have been tested once the sixteen warps meet here: if every one of them is retained, the head is left to
+      // the one-pass kernel
       asm volatile("bar.sync 1, 512;" ::: "memory");
-      if (st < G) {
-        int got = 0;
-        for (int x = 0; x < 2 * wpad; ++x) got += __popc(rowmask[st * 2 * wpad + x]);
-        int want = 0;
-        for (int i = i0a; i < T; i += kScoutSampleStride)
-          for (int e = 0; e < 2; ++e)
-            if (i + e < T) want += (i + e >= i0b) ? 2 : 1;
-        dflag[st] = (got == want);
+      if (st < 32) {
+        int got = 0, want = 0;
+        for (int x = st; x < KB * wpad; x += 32) got += __popc(rowmask[x]);
+        for (int i = i0 + st * kScoutSampleStride; i < T; i += 32 * kScoutSampleStride)
+          for (int e = i; e < min(i + 2, T); ++e)
+            for (int kb = 0; kb < nkb; ++kb) want += e >= first(ja + kb);
+        for (int sft = 16; sft > 0; sft >>= 1) {
+          got += __shfl_xor_sync(0xffffffffu, got, sft);
+          want += __shfl_xor_sync(0xffffffffu, want, sft);
+        }
+        if (st == 0) *(volatile int*)&direct_s = (got == want);
       }
       asm volatile("bar.sync 1, 512;" ::: "memory");
       if (st == 0) mbar_arrive(&phase_bar);
       return true;
     });
-    // every tile has been tested once the sixteen warps meet here: the rows go out
+    // every tile has been tested once the sixteen warps meet here: the rows go out, one warp per row
     asm volatile("bar.sync 1, 512;" ::: "memory");
-    for (int r = (st >> 5); r < G * 2; r += 16) {           // one warp per row
-      const int h = r >> 1, kb = r & 1, j = ja + kb;
-      if (j >= p.Tk) continue;
-      const bool direct = sampling && dflag[h] != 0;
-      const size_t orow = out_row0 + (size_t)h * p.Tk + j;
+    const int kb = st >> 5, j = ja + kb;
+    if (kb < KB && j < p.Tk) {
+      const bool direct = sampling && direct_s != 0;
       uint32_t pop = 0;
       for (int x = lane; x < wpad; x += 32) {
-        const uint32_t wv = direct ? 0u : rowmask[r * wpad + x];
-        p.mask[orow * wpad + x] = wv;
-        if (!direct && p.tel_bitmask && x < p.words) p.tel_bitmask[orow * p.words + x] = wv;
+        const uint32_t wv = direct ? 0u : rowmask[kb * wpad + x];
+        p.mask[(out_row + kb) * wpad + x] = wv;
+        if (!direct && p.tel_bitmask && x < p.words) p.tel_bitmask[(out_row + kb) * p.words + x] = wv;
         pop += __popc(wv);
       }
       for (int sft = 16; sft > 0; sft >>= 1) pop += __shfl_xor_sync(0xffffffffu, pop, sft);
       if (lane == 0) {
-        p.row_count[orow] = direct ? kScoutDirectRow : pop;
-        const bool present = kb ? has_b : true;
+        p.row_count[out_row + kb] = direct ? kScoutDirectRow : pop;
         if (!direct) {
-          if (p.tel_retained) p.tel_retained[orow] = pop;
-          if (p.totals && present) {
+          if (p.tel_retained) p.tel_retained[out_row + kb] = pop;
+          if (p.totals && kb < nkb) {
             atomicAdd(&p.totals[0], (unsigned long long)pop);
-            atomicAdd(&p.totals[1], (unsigned long long)(kb ? max(T - i0b, 0) : ni));
+            atomicAdd(&p.totals[1], (unsigned long long)max(T - first(j), 0));
           }
         }
       }

@@ -78,6 +78,36 @@ def test_bwd_one_or_two_passes(mala, oracle, N, d, Hq, Hkv, tau):
     _run_isolated(mala, oracle, w, tau)
 
 
+@pytest.mark.parametrize("N,d,Hq,Hkv", [(520, 128, 147, 49), (520, 128, 148, 37), (600, 64, 160, 40), (385, 64, 148, 74)])
+def test_bwd_first_pass_of_two_or_four_key_blocks(mala, oracle, N, d, Hq, Hkv):
+    # on a GPU of 148 SMs the first pass takes four key blocks per CTA from 296 CTAs on; ragged last blocks and pairs
+    w = W.custom_prefill(1, Hq, Hkv, N, d, head_types=["diffuse", "peaked"] * (Hq // 2) + ["peaked"] * (Hq % 2), seed=N, preset="R")
+    r = _run_isolated(mala, oracle, w, 1e-3)
+    assert r["skipped"] > 0
+
+
+def test_bwd_first_pass_long_rows(mala, oracle):
+    # so many query blocks (2057) that the masks of a CTA leave room for two Q tiles instead of three; sampled key blocks
+    N = 263200
+    w = W.custom_prefill(1, 1, 1, N, 128, head_types=["peaked"], seed=5, preset="S", device="cuda")
+    q, k, v, do = (w[x] for x in ("q", "k", "v", "do"))
+    o, lse, _ = mala.fwd(q, k, v, w["scale"], 1e-4)
+    dq, dk, dv, st = mala.bwd(q, k, v, o, do, lse, w["scale"], 1e-4, stats=True)
+    torch.cuda.synchronize()
+    assert mala.device_status() == 0
+    units = [(0, 0, 1601), (0, 0, 2056)]
+    ref = oracle.bwd(*(x.cpu() for x in (q, k, v)), o.float().cpu(), do.cpu(), lse.cpu().numpy(), w["scale"], 1e-4, 128, 128,
+                     key_units=units)
+    gm = st.mask(2057)[0, 0].cpu().numpy()
+    for _, _, j in units:
+        om, oc = ref["mask"][0, 0, j], ref["crit"][0, 0, j]
+        differ = gm[j] != (om == 2)
+        assert (np.abs(oc[differ]) <= parity.MASK_BAND).all()
+        rows = slice(j * 128, min(N, (j + 1) * 128))
+        parity.check_grad(dk[0, rows, 0].float().cpu().numpy(), ref["dk"][0, rows, 0], f"dk block {j}")
+        parity.check_grad(dv[0, rows, 0].float().cpu().numpy(), ref["dv"][0, rows, 0], f"dv block {j}")
+
+
 @pytest.mark.parametrize("tau", [1e-5, 1e-4, 1e-3, 1.0])
 @pytest.mark.parametrize("N,d", [(1024, 128), (1000, 128), (1024, 64)])
 def test_bwd_skipping_regime(mala, oracle, N, d, tau):
