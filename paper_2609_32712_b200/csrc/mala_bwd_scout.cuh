@@ -37,8 +37,12 @@
 namespace mala {
 
 constexpr uint32_t kScoutDirectRow = 0xffffffffu;   // row_count of a row left to the one-pass kernel
-constexpr int kScoutSampleStride = 16;              // two tiles of every sixteen of a row are sampled first ...
-constexpr int kScoutSampleMinTiles = 32;            // ... in rows of at least this many tiles
+// Two tiles of every sixteen of a row are sampled first in rows of at least 32 tiles, in calls with at least 96 query blocks (192 with
+// 64 columns).  Below that the rows that retain everything go with the list: one kernel with one tail instead of two, and every
+// tile tested, against a kernel that tests as it goes (whole backward, 16 / 4 heads, sampled / not: 8192 tokens, every tile retained
+// 1.07 / 0.99 ms, a third 0.45 / 0.47; 16384 tokens 3.42 / 3.69, 1.43 / 1.43; 64 columns, 16384 tokens, 8 heads 1.35 / 1.16).
+constexpr int kScoutSampleStride = 16;
+constexpr int kScoutSampleMinTiles = 32;
 
 struct ScoutParams {
   const float* bq;            // [B,Hq,Np] lse2 + log2(tau / L_q); +inf on padding rows

@@ -158,16 +158,20 @@ __device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontro
 // Launches `kernel`, which begins with wait_for_primary(), as a programmatic dependent of the kernel before it.  A launch that
 // fails is reported here alone: the runtime's last error is taken back, so that the next call's check does not meet it.
 template <typename... P, typename... A>
-inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+inline cudaError_t launch_dependent_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = stream;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = stream; cfg.dynamicSmemBytes = smem;
   cfg.attrs = at; cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
   if (e != cudaSuccess) (void)cudaGetLastError();
   return e;
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, const A&... args) {
+  return launch_dependent_smem(kernel, grid, block, 0, stream, args...);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -86,6 +86,34 @@ def test_bwd_first_pass_of_two_or_four_key_blocks(mala, oracle, N, d, Hq, Hkv):
     assert r["skipped"] > 0
 
 
+@pytest.mark.parametrize("T,d", [(95, 128), (96, 128), (191, 64), (192, 64)])
+def test_bwd_with_and_without_samples(mala, oracle, T, d):
+    # just below and at the length from which rows that retain everything are left to the one-pass kernel, which then adds to the
+    # dK, dV of the list (a diffuse and a peaked head share them): key blocks with rows of more and of fewer than 32 tiles
+    N = T * 128 - 9
+    w = W.custom_prefill(1, 2, 1, N, d, head_types=["diffuse", "peaked"], seed=T, preset="R", device="cuda")
+    q, k, v, do = (w[x] for x in ("q", "k", "v", "do"))
+    o, lse, _ = mala.fwd(q, k, v, w["scale"], 1e-4)
+    dq, dk, dv, st = mala.bwd(q, k, v, o, do, lse, w["scale"], 1e-4, stats=True)
+    torch.cuda.synchronize()
+    assert mala.device_status() == 0
+    units, rows_of = [(0, 0, 3), (0, 0, T - 40), (0, 0, T - 20), (0, 0, T - 1)], [(0, 0, T // 2), (0, 1, T - 1)]
+    ref = oracle.bwd(*(x.cpu() for x in (q, k, v)), o.float().cpu(), do.cpu(), lse.cpu().numpy(), w["scale"], 1e-4, 128, 128,
+                     key_units=units, dq_units=rows_of)
+    gm = st.mask(T)[0].cpu().numpy()
+    for _, _, j in units:
+        for h in range(2):
+            om, oc = ref["mask"][0, h, j], ref["crit"][0, h, j]
+            differ = gm[h, j] != (om == 2)
+            assert (np.abs(oc[differ]) <= parity.MASK_BAND).all()
+        rows = slice(j * 128, min(N, (j + 1) * 128))
+        parity.check_grad(dk[0, rows, 0].float().cpu().numpy(), ref["dk"][0, rows, 0], f"dk block {j}")
+        parity.check_grad(dv[0, rows, 0].float().cpu().numpy(), ref["dv"][0, rows, 0], f"dv block {j}")
+    for _, h, i in rows_of:
+        rows = slice(i * 128, min(N, (i + 1) * 128))
+        parity.check_grad(dq[0, rows, h].float().cpu().numpy(), ref["dq"][0, rows, h], f"dq block {i}")
+
+
 def test_bwd_first_pass_long_rows(mala, oracle):
     # so many query blocks (2057) that the masks of a CTA leave room for two Q tiles instead of three; sampled key blocks
     N = 263200
