@@ -155,7 +155,7 @@ mala_fwd_one_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   };
 
   if (tid == 0) {
-    ctl.early_exit = (*(volatile int*)status != 0) || (smem_u32(smem) & 1023u) != 0;
+    ctl.early_exit = (*(volatile int*)status != 0);
     mbar_init(&q_full, 1);
     for (int s = 0; s < KS; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1); }
     for (int s = 0; s < VS; ++s) { mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1); }
