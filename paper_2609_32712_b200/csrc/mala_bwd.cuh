@@ -127,6 +127,7 @@ struct ListIter {
 };
 
 constexpr int kBwdListWords = 2048;   // mask words of one CTA's G rows held in shared memory (list mode)
+constexpr int kBwdListHeads = 16;     // query heads of a group in the two-pass path (the one-pass kernel alone takes any number)
 
 // kList (with kDense): the tiles are those of the mask rows in p.list_mask, all of them retained: no test, no votes,
 // the dense tile pipeline on a sparse tile sequence.
@@ -219,17 +220,22 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     }
   }
 
-  // the query heads of the group this CTA handles: all of them, or (one-pass kernel behind the first pass) those whose
-  // rows the first pass left alone
-  __shared__ int hsel[16];
+  // the query heads of the group this CTA handles: all of them, however many, or (one-pass kernel behind the first pass, which
+  // takes groups of up to kBwdListHeads) those whose rows the first pass left alone
+  __shared__ int hsel[kBwdListHeads];
   __shared__ int nsel_s;
-  if (warp == 0) {   // (one row flag per lane)
-    bool mine = lane < G && lane < 16;
-    if (!kList && !kDense && p.sel_rows)
-      mine = mine && __ldg(p.sel_rows + ((size_t)b * p.Hq + (size_t)hkv * G + lane) * p.Tk + j) == 0xffffffffu;
-    const uint32_t m = __ballot_sync(0xffffffffu, mine);
-    if (mine) hsel[__popc(m & ((1u << lane) - 1u))] = lane;
-    if (lane == 0) nsel_s = __popc(m);
+  const bool some_heads = !kList && !kDense && p.sel_rows;
+  auto head = [&](int x) -> int { return some_heads ? hsel[x] : x; };   // the x-th handled head of the group
+  if (warp == 0) {
+    if (some_heads) {   // (one row flag per lane)
+      const bool mine = lane < G && lane < kBwdListHeads &&
+                        __ldg(p.sel_rows + ((size_t)b * p.Hq + (size_t)hkv * G + lane) * p.Tk + j) == 0xffffffffu;
+      const uint32_t m = __ballot_sync(0xffffffffu, mine);
+      if (mine) hsel[__popc(m & ((1u << lane) - 1u))] = lane;
+      if (lane == 0) nsel_s = __popc(m);
+    } else if (lane == 0) {
+      nsel_s = G;
+    }
   }
   if (tid == 0) {
     early_exit = (*(volatile int*)status != 0);
@@ -275,7 +281,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (int n = 0; n < n_tot && ok; ++n, ++i) {
         if (kList) it.next(hk, i);
         else if (i == T) { i = i0; ++hk; }
-        const int hq = hkv * G + (kList ? hk : hsel[hk]);
+        const int hq = hkv * G + (kList ? hk : head(hk));
         const int s = n & 1;
         ok = mbar_wait(&q_empty[s], ((n >> 1) & 1) ^ 1, status);
         if (!ok) break;
@@ -451,7 +457,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     // per-query vectors of tile 0 into slot 0 (published by the first column quarter), then a group sync
     if (qt == 0) {
       if (!kDense && p.behind == kBehindPre) wait_for_primary();
-      const size_t x = vec_index(kList ? h_nx : hsel[0], kList ? i_nx : i0);
+      const size_t x = vec_index(kList ? h_nx : head(0), kList ? i_nx : i0);
       vec[0][0][rl] = p.lse2[x];
       vec[0][1][rl] = p.bq[x];
       vec[0][2][rl] = p.Dq[x];
@@ -469,7 +475,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // prefetch the per-query vectors of the next tile
       float nx0 = 0.f, nx1 = 0.f, nx2 = 0.f;
       if (qt == 0 && n + 1 < n_tot) {
-        const size_t x = kList ? vec_index(h_nx, i_nx) : (last_of_head ? vec_index(hsel[hq_n + 1], i0) : vec_index(hsel[hq_n], i + 1));
+        const size_t x = kList ? vec_index(h_nx, i_nx) : (last_of_head ? vec_index(head(hq_n + 1), i0) : vec_index(head(hq_n), i + 1));
         nx0 = p.lse2[x]; nx1 = p.bq[x]; nx2 = p.Dq[x];
       }
       ok = mbar_wait_warp(&s_full, n & 1, status);
@@ -532,7 +538,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (stat_thread) {
           ++r_head;
           if (p.bitmask) {
-            uint32_t* bm_row = p.bitmask + ((size_t)(b * p.Hq + hkv * G + hsel[hq_n]) * p.Tk + j) * p.words;
+            uint32_t* bm_row = p.bitmask + ((size_t)(b * p.Hq + hkv * G + head(hq_n)) * p.Tk + j) * p.words;
             if ((i >> 5) != bm_word) {
               if (bm_word >= 0) bm_row[bm_word] = bm_bits;
               bm_word = i >> 5;
@@ -603,7 +609,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         ++r;
       }
       if (stat_thread && last_of_head) {   // last tile of this query head
-        const size_t row = (size_t)(b * p.Hq + hkv * G + hsel[hq_n]) * p.Tk + j;
+        const size_t row = (size_t)(b * p.Hq + hkv * G + head(hq_n)) * p.Tk + j;
         if (p.bitmask && bm_word >= 0) p.bitmask[row * p.words + bm_word] = bm_bits;
         if (p.retained) p.retained[row] = (uint32_t)r_head;
         if (p.totals) {
@@ -683,7 +689,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (info < 0) break;
       const int n = info >> 1, ds = info & 1;
       // (the tile's coordinates while the dQ MMAs are still running: the announcement precedes their completion)
-      int hq = hkv * G + hsel[n / ni], i = i0 + n % ni;
+      int hq = hkv * G + head(n / ni), i = i0 + n % ni;
       if (kList) { int hl; it.next(hl, i); hq = hkv * G + hl; }   // (every tile of the list is announced, in order)
       const int tile = p.cu ? (int)((size_t)hq * (p.Np / 128) + (size_t)(prow0 / 128 + i))
                             : (int)(((size_t)b * p.Hq + hq) * p.T + (size_t)i);
@@ -992,7 +998,7 @@ inline int bwd_launch(mala_tin q, mala_tin k, mala_tin v, mala_tin o, mala_tin d
   // (whole backward, 1024 tokens, 2 heads of 64 columns: 27.7 us instead of 39.8, 29.9 instead of 42.2 with 128 columns and
   // nearly every tile skipped; 512 tokens, 32 / 8 heads: 61 instead of 87).
   const bool brief = (long long)Tk * Hkv * B <= sms && (Hq / Hkv) * T <= 16;
-  const bool two_pass = !dense && !brief && MALA_BWD_TWO_PASS && (Hq / Hkv) * wpad <= kBwdListWords && (Hq / Hkv) <= 16 &&
+  const bool two_pass = !dense && !brief && MALA_BWD_TWO_PASS && (Hq / Hkv) * wpad <= kBwdListWords && (Hq / Hkv) <= kBwdListHeads &&
                         ws_bytes >= base_bytes + bwd_list_bytes(B, Hq, T, Tk);
   int rc;
   // (Where every key block has an SM: 1024 tokens, 2 heads of 64 columns, the whole backward 33 -> 28 us, 512 tokens 25 -> 19.)

@@ -78,6 +78,15 @@ def test_bwd_one_or_two_passes(mala, oracle, N, d, Hq, Hkv, tau):
     _run_isolated(mala, oracle, w, tau)
 
 
+@pytest.mark.parametrize("tau", [0.0, 1e-3])
+@pytest.mark.parametrize("B,N,d,Hq,Hkv", [(1, 300, 128, 16, 1), (1, 300, 128, 17, 1), (1, 640, 64, 33, 1), (38, 250, 64, 34, 2)])
+def test_bwd_groups_of_more_than_sixteen_heads(mala, oracle, B, N, d, Hq, Hkv, tau):
+    # the two-pass path ends at sixteen query heads per KV head; the kernel that walks all heads of a group takes any number
+    # (the last case: more key blocks than a GPU of 148 SMs has SMs)
+    w = W.custom_prefill(B, Hq, Hkv, N, d, head_types=["diffuse", "peaked"] * (Hq // 2) + ["peaked"] * (Hq % 2), seed=N, preset="R")
+    _run_isolated(mala, oracle, w, tau)
+
+
 @pytest.mark.parametrize("N,d,Hq,Hkv", [(520, 128, 147, 49), (520, 128, 148, 37), (600, 64, 160, 40), (385, 64, 148, 74)])
 def test_bwd_first_pass_of_two_or_four_key_blocks(mala, oracle, N, d, Hq, Hkv):
     # on a GPU of 148 SMs the first pass takes four key blocks per CTA from 296 CTAs on; ragged last blocks and pairs

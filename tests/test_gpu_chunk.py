@@ -165,6 +165,12 @@ def test_chunk_backward_from_any_position_literal(mala, oracle, Nk, Nq, d, Hq, H
     _run_bwd_any_offset(mala, oracle, _chunk(w, Nq), tau)
 
 
+@pytest.mark.parametrize("tau", [0.0, 1e-4])
+def test_chunk_backward_group_of_more_than_sixteen_heads(mala, oracle, tau):
+    w = W.custom_prefill(1, 20, 1, 700, 128, seed=700)
+    _run_bwd_any_offset(mala, oracle, _chunk(w, 333), tau)
+
+
 @pytest.mark.parametrize("tau", [1e-4, 1.0])
 @pytest.mark.parametrize("Nk,Nq,d", [(2000, 555, 128), (2500, 1300, 64)])
 def test_chunk_backward_from_any_position_skipping_regime(mala, oracle, Nk, Nq, d, tau):

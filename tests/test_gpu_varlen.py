@@ -81,6 +81,11 @@ def test_varlen_literal(mala, oracle, lens, Hq, Hkv, d, tau):
     _run(mala, oracle, lens, Hq, Hkv, d, tau)
 
 
+@pytest.mark.parametrize("tau", [0.0, 1e-4])
+def test_varlen_group_of_more_than_sixteen_heads(mala, oracle, tau):
+    _run(mala, oracle, [333, 1, 517], 17, 1, 64, tau)
+
+
 @pytest.mark.parametrize("tau", [1e-4, 1.0])
 def test_varlen_skipping_regime(mala, oracle, tau):
     sk = _run(mala, oracle, [1024, 300, 1500, 777], 4, 2, 128, tau, preset="R",
