@@ -148,7 +148,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint8_t* sDS = (D == 128) ? sDO : sDO + 2 * Cfg::kTileBytes;
 
   __shared__ uint64_t kv_full, q_full[2], q_empty[2], do_full[2], do_empty[2], s_full, vote_bar[2], p_full, dp_full,
-      ds_full, dst_full, dv_done, dq_full, dq_empty, dq_info_bar, grp_bar, fin_bar, stg_full, ds_free;
+      ds_full, dst_full, dv_done, dq_full, dq_empty, dq_info_bar, grp_bar, fin_bar, stg_full, ds_free[2];
   __shared__ __align__(16) float vec[3][3][128];   // [slot][lse2 | bq | Dq][query column]
   __shared__ uint32_t tmem_base_s;
   __shared__ int flag[3];
@@ -248,7 +248,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     mbar_init(&s_full, 1); mbar_init(&p_full, 16); mbar_init(&dp_full, 1); mbar_init(&ds_full, 16); mbar_init(&dst_full, 16);
     mbar_init(&dv_done, 1); mbar_init(&grp_bar, 16); mbar_init(&dq_full, 1); mbar_init(&dq_empty, 4); mbar_init(&dq_info_bar, 1);
     mbar_init(&fin_bar, 1);
-    mbar_init(&stg_full, 4); mbar_init(&ds_free, 1);
+    mbar_init(&stg_full, 4); mbar_init(&ds_free[0], 1); mbar_init(&ds_free[1], 1);
     flag[0] = flag[1] = flag[2] = 0;
     dq_info = -1;
     mbar_fence_init();
@@ -406,7 +406,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             *(volatile int*)&dq_info = n * 2 + ds;
             mbar_arrive(&dq_info_bar);
             tc_commit(&dq_full);
-            tc_commit(&ds_free);   // dS^T has been consumed: the dQ group may stage the dQ tile in that stage
+            tc_commit(&ds_free[r & 1]);   // dS^T has been consumed: the dQ group may stage the dQ tile in that stage
           }
           ++r;
         } else {
@@ -714,7 +714,11 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           for (int v = 0; v < 8; ++v)
             red_add_v4(acc + (c * 8 + v) * 512, a[c][4 * v], a[c][4 * v + 1], a[c][4 * v + 2], a[c][4 * v + 3]);
       }
-      ok = mbar_wait_warp(&ds_free, k & 1, status);     // dQ and dK have consumed dS^T: its stage may be overwritten
+      // dQ and dK have consumed dS^T: its stage may be overwritten.  Two barriers in turn, because dq_empty has been given: while
+      // this warp is still at its reductions, the issuer may complete the next tile's phase (the one after that needs this
+      // warp's next dq_empty), and a wait on one barrier for both would then never see its own parity again.  (dq_full has said
+      // the same; without this wait 64 columns are 1 % slower, the copies into the stage meeting the score group's.)
+      ok = mbar_wait_warp(&ds_free[k & 1], (k >> 1) & 1, status);
       if (!ok) break;
 #pragma unroll
       for (int c = D / 64; c < D / 32; ++c) {
