@@ -396,10 +396,11 @@ mala_fwd_one_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (!kDense) {
         // Eq. 3: skip iff rowmax - (m + log l) < log(tau / L) for every valid row (nothing retained yet: lg = -inf)
         const bool any = __any_sync(0xffffffffu, valid && !((mt - lg) - theta < 0.f));
+        tc_fence_before();
+        __syncwarp();       // (a vote orders no memory: all lanes' letters and reads of the scores stand before the arrival)
         if (lane == 0) {
           if (any) *(volatile int*)&flag[t & 3] = 1;
           if (warp == 4) *(volatile int*)&flag[(t + 2) & 3] = 0;   // (last read for tile t - 2, next set for tile t + 2)
-          tc_fence_before();
           mbar_arrive(&vote_bar[x]);
         }
         // A warp that found a retaining row knows the outcome and goes straight on.
@@ -409,7 +410,7 @@ mala_fwd_one_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           retain = __all_sync(0xffffffffu, (*(volatile int*)&flag[t & 3]) != 0);
         }
         if (!retain) {
-          if (!fresh) *in_box = ~0ull;        // (both halves have voted, so the letter is there)
+          if (!fresh) *in_box = ~0ull;        // (both halves have voted behind their letters, so it is there)
           fresh = false;
           continue;
         }
