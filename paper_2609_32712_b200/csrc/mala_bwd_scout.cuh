@@ -270,8 +270,9 @@ mala_bwd_scout_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           vote = fmaf(fmaxf(max3(m0, m1, m2), m3), c2, -need) >= 0.f;   // Eq. 4 (padding rows: need = +inf)
         }
         const bool any = __any_sync(0xffffffffu, vote);
+        tc_fence_before();
+        __syncwarp();       // (all lanes' reads of the buffer stand before the arrival)
         if (lane == 0) {
-          tc_fence_before();
           mbar_arrive(&s_empty[buf]);
           if (any) atomicOr(&rowmask[kb * wpad + (i >> 5)], 1u << (i & 31));
         }
