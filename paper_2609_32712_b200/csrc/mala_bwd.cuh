@@ -520,10 +520,11 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (!kDense) {
         const bool vote = valid_key && !(crit < 0.f);
         const bool any = __any_sync(0xffffffffu, vote);
+        tc_fence_before();
+        __syncwarp();       // (all lanes' reads of the scores stand before the arrival)
         if (lane == 0) {
           if (any) *(volatile int*)&flag[slot] = 1;
           if (warp == 4) *(volatile int*)&flag[slot == 2 ? 0 : slot + 1] = 0;
-          tc_fence_before();
           mbar_arrive(&vote_bar[n & 1]);
         }
         // A warp that found a retained entry knows the outcome (the vote is an OR) and goes straight on; a warp

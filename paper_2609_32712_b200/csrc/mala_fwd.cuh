@@ -458,10 +458,11 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // Eq. 3: skip iff rowmax - (m + log l) < log(tau / L) for every valid row
         const bool vote = valid && !((mt - lg) - theta < 0.f);   // (nothing retained yet: lg = -inf)
         const bool any = __any_sync(0xffffffffu, vote);
+        tc_fence_before();
+        __syncwarp();       // (all lanes' reads of the scores stand before the arrival)
         if (lane == 0) {
           if (any) *(volatile int*)&flag[x][t % 3] = 1;
           if ((warp & 3) == 0) *(volatile int*)&flag[x][(t + 1) % 3] = 0;
-          tc_fence_before();
           mbar_arrive(&vote_bar[x]);
         }
         // A warp that found a retaining row knows the outcome (the vote is an OR) and goes straight on; only a warp
