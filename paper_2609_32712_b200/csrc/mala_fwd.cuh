@@ -408,7 +408,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const bool mask_first = x ? (hB == dB) : (hA == dA);
     // (l: sum of the keys 0-63 of the tiles, and of the keys 64-127 -- in this order, because mala_fwd_one_kernel has a thread for
     // either, and a row comes out the same bit for bit whichever kernel its call takes)
-    float m_ref = -INFINITY, l0 = 0.f, l1 = 0.f, l = 0.f, lg = -INFINITY;
+    float m_ref = -INFINITY, l0 = 0.f, l1 = 0.f, lg = -INFINITY;
     int r = 0;
     bool ok = true;
     uint32_t bm_bits = 0;
@@ -419,6 +419,13 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
     for (int t = 0; t < T; ++t) {
       const int j = j0 - first - t;
+      // The row's normalizer so far, as the test needs it: here, beside the wait for the scores, with 64 columns, and behind the
+      // sums below with 128 (1300 tokens, 32 heads of 64: 27.6 us, there 28.2; 2360 tokens, 16 heads of 128, every tile retained:
+      // 49.2 us, here 50.6 -- but with nearly every tile skipped 34.1, here 32.5).
+      if constexpr (!kDense && D == 64) {
+        lg = m_ref + __log2f(l0 + l1);
+        asm volatile("" : "+f"(lg));
+      }
       ok = mbar_wait_warp(&s_full[x], t & 1, status);
       if (!ok) break;
       tc_fence_after();
@@ -567,8 +574,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       MALA_P_CHUNK(s3, 48)
 #undef MALA_P_CHUNK
       l1 += (sum0 + sum1) + (sum2 + sum3);
-      l = l0 + l1;
-      if (!kDense) lg = m_ref + __log2f(l);
+      if constexpr (!kDense && D != 64) lg = m_ref + __log2f(l0 + l1);
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
@@ -576,6 +582,7 @@ mala_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       ++r;
     }
 
+    const float l = l0 + l1;
     if (ok && present_x) {
       // finalize once every PV has retired: O <- O / l, lse <- m + log l
       ok = mbar_wait_warp(&fin_bar, 0, status);
