@@ -316,7 +316,7 @@ mala_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // (dense, 128 columns: 0.7-1.0 % faster with the slower way to wait, 23.5 against 23.7 ms at 32K and 32 / 8 heads; with the
       // test, in the list mode and with 64 columns the quick one is 1.5-6 % faster)
       auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-        if constexpr (kDense && !kList && D == 128) return __all_sync(0xffffffffu, mbar_wait(bar, parity, status));
+        if constexpr (kDense && !kList && D == 128) return mbar_wait_then_vote(bar, parity, status);
         else return mbar_wait_warp(bar, parity, status);
       };
       constexpr uint32_t idesc_s = make_idesc_bf16(128, 128, false, false);    // S^T, dP^T

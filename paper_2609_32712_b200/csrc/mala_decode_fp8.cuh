@@ -88,6 +88,11 @@ struct DecF8Params {
 // kSplit_: five to eight query heads per KV head.  A stream's softmax group is then eight warps, two threads per key:
 // warps 0-3 carry the heads 0-3 through the chain and warps 4-7 the heads 4-7 (both read the same TMEM lanes, their
 // own columns), so that a thread's chain is as long as with four heads; the two halves only meet in the tile's vote.
+// Two kinds of wait: the softmax groups, whose waits are the streams' chain, use mbar_wait_warp; the issuing warps, which share
+// their schedulers and wait most of the time, and the epilogue group mbar_wait_then_vote, and so do the eight warps of a split group
+// for one another.  (With mbar_wait_warp everywhere: 64 / 8 heads, 21 sequences of up to 5135 keys, pages of 16: 52.3 us instead of
+// 50.0; 32 / 8 heads, 2 of up to 60000, pages of 64: 66.5 instead of 64.3; with the other one everywhere 16 sequences of up to
+// 40000 keys, 32 / 8 heads, take 148.8 instead of 146.9.)
 template <int NG_, bool kDense_, bool kSplit_ = false>
 struct DecF8Cfg {
   static constexpr int kRawBytes = 128 * 128;            // one e4m3 tile
@@ -312,7 +317,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         if (T == 0) continue;
         int b, hkv, split, j0;
         geometry(item, b, hkv, split, j0, T);
-        if (ne >= 1) ok = mbar_wait_warp(&qr_free[k], (uint32_t)((ne - 1) & 1), status);
+        if (ne >= 1) ok = mbar_wait_then_vote(&qr_free[k], (uint32_t)((ne - 1) & 1), status);
         if (!ok) break;
         if (lane == 0) {
           mbar_arrive_expect_tx(&qr_full[k], (uint32_t)R * 128u * 2u);
@@ -324,7 +329,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           const uint32_t ph = (uint32_t)((g / NK) & 1);
           const int x = (j0 - t) * p.ppt + lane;   // (a table entry past the row's end reads as "no page": zeros)
           const int pg = (lane < p.ppt && x < p.max_pages) ? __ldg(p.block_table + (size_t)b * p.max_pages + x) : -1;
-          ok = mbar_wait_warp(&kr_empty[k][s], ph ^ 1u, status);
+          ok = mbar_wait_then_vote(&kr_empty[k][s], ph ^ 1u, status);
           if (!ok) break;
           if (lane < 8) t_page[k][g & 7][lane] = pg;
           __syncwarp();
@@ -332,7 +337,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           __syncwarp();
           if (lane < p.ppt) tma_load_4d(sKr + s * RB + lane * p.prows * 128, &tmK, &kr_full[k][s], 0, 0, hkv, pg);
           if (kDense) {
-            ok = mbar_wait_warp(&v_empty[k][s], ph ^ 1u, status);
+            ok = mbar_wait_then_vote(&v_empty[k][s], ph ^ 1u, status);
             if (!ok) break;
             if (lane == 0) mbar_arrive_expect_tx(&v_full[k][s], RB);
             __syncwarp();
@@ -395,8 +400,8 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         // the item's queries have landed: row qh (128 bf16 in two 64-column panels, rows qh and HALF + qh of the
         // landing buffer; lane = four consecutive columns) becomes rows qh and HALF + qh of the e4m3 operand, once the
         // MMAs of the item that had the operand's slot before have read it
-        ok = mbar_wait_warp(&qr_full[k], (uint32_t)(ne & 1), status);
-        if (ok && ne >= 2) ok = mbar_wait_warp(&q8_free[k][ip], (uint32_t)(((ne >> 1) - 1) & 1), status);
+        ok = mbar_wait_then_vote(&qr_full[k], (uint32_t)(ne & 1), status);
+        if (ok && ne >= 2) ok = mbar_wait_then_vote(&q8_free[k][ip], (uint32_t)(((ne >> 1) - 1) & 1), status);
         if (!ok) break;
         for (int qh = 0; qh < R; ++qh) {
           const int e0 = lane * 4;
@@ -425,11 +430,11 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         for (int t = 0; t < T && ok; ++t, ++g) {
           const int sb = g & 3, kc = g % NK;
           if (g >= 4) {
-            ok = mbar_wait_warp(&s_free[k][sb], (uint32_t)(((g >> 2) - 1) & 1), status);
+            ok = mbar_wait_then_vote(&s_free[k][sb], (uint32_t)(((g >> 2) - 1) & 1), status);
             // (the vote of the tile that had this slot has been read: its flag may be overwritten)
-            if (!kDense && ok) ok = mbar_wait_warp(&vote_read[k][sb], (uint32_t)(((g >> 2) - 1) & 1), status);
+            if (!kDense && ok) ok = mbar_wait_then_vote(&vote_read[k][sb], (uint32_t)(((g >> 2) - 1) & 1), status);
           }
-          if (ok) ok = mbar_wait_warp(&kr_full[k][kc], (uint32_t)((g / NK) & 1), status);
+          if (ok) ok = mbar_wait_then_vote(&kr_full[k][kc], (uint32_t)((g / NK) & 1), status);
           if (!ok) break;
           if constexpr (kSmall) {   // one pair of scales per page of the tile, and the largest V scale
             const int pg = lane < 8 ? *(volatile int*)&t_page[k][g & 7][lane] : -1;
@@ -480,8 +485,8 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           int b, hkv, split, j0;
           geometry(item, b, hkv, split, j0, T);
           for (int t = 0; t < T && ok; ++t, ++g) {
-            ok = mbar_wait_warp(&vote_bar[k][g & 3], (uint32_t)((g >> 2) & 1), status);
-            if (ok && g >= 8) ok = mbar_wait_warp(&ret_free[k][g & 7], (uint32_t)(((g >> 3) - 1) & 1), status);
+            ok = mbar_wait_then_vote(&vote_bar[k][g & 3], (uint32_t)((g >> 2) & 1), status);
+            if (ok && g >= 8) ok = mbar_wait_then_vote(&ret_free[k][g & 7], (uint32_t)(((g >> 3) - 1) & 1), status);
             if (!ok) break;
             const bool retain = __shfl_sync(0xffffffffu, *(volatile int*)&flag[k][0][g & 7] |
                                                                   (kSplit ? *(volatile int*)&flag[k][1][g & 7] : 0), 0) != 0;
@@ -489,7 +494,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             if (leader) mbar_arrive(&vote_read[k][g & 3]);
             if (retain) {
               const int vs = nv % NV;
-              if (nv >= NV) ok = mbar_wait_warp(&v_empty[k][vs], (uint32_t)(((nv / NV) - 1) & 1), status);
+              if (nv >= NV) ok = mbar_wait_then_vote(&v_empty[k][vs], (uint32_t)(((nv / NV) - 1) & 1), status);
               if (!ok) break;
               if constexpr (kSmall) {
                 if (lane == 0) mbar_arrive_expect_tx(&v_full[k][vs], RB);
@@ -527,7 +532,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         for (int t = 0; t < T && ok; ++t, ++g) {
           bool retain = true;
           if (!kDense) {
-            ok = mbar_wait_warp(&ret_full[k][g & 7], (uint32_t)((g >> 3) & 1), status);
+            ok = mbar_wait_then_vote(&ret_full[k][g & 7], (uint32_t)((g >> 3) & 1), status);
             if (!ok) break;
             retain = __shfl_sync(0xffffffffu, *(volatile int*)&ret_ring[k][g & 7], 0) != 0;
             __syncwarp();
@@ -535,10 +540,10 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           }
           if (retain) {
             const int ps = npv % PP, vc = npv % NV;
-            ok = mbar_wait_warp(&p_full[k][ps], (uint32_t)((npv / PP) & 1), status);
-            if (ok) ok = mbar_wait_warp(&v_full[k][vc], (uint32_t)((npv / NV) & 1), status);
+            ok = mbar_wait_then_vote(&p_full[k][ps], (uint32_t)((npv / PP) & 1), status);
+            if (ok) ok = mbar_wait_then_vote(&v_full[k][vc], (uint32_t)((npv / NV) & 1), status);
             // (the accumulator is that of the item two before, which has to have been written out)
-            if (ok && r_item == 0 && ne >= 2) ok = mbar_wait_warp(&o_free[k][ip], (uint32_t)(((ne >> 1) - 1) & 1), status);
+            if (ok && r_item == 0 && ne >= 2) ok = mbar_wait_then_vote(&o_free[k][ip], (uint32_t)(((ne >> 1) - 1) & 1), status);
             if (!ok) break;
             tc_fence_after();
             const uint32_t dO = tO + (uint32_t)ip * 16u;
@@ -558,7 +563,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       }
       if (leader) tc_commit(&fin_bar[k]);
       __syncwarp();
-      mbar_wait_warp(&fin_bar[k], 0, status);
+      mbar_wait_then_vote(&fin_bar[k], 0, status);
     }
     if (!ok) { const long long t0 = clock64(); while (clock64() - t0 < 400000) {} }
   } else if (warp >= 4 * NG + 4 * NG * HS) {
@@ -602,8 +607,8 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
 #pragma unroll
       for (int i = 0; i < NG; ++i) if (i == k) { ne = ne_k[i]; ++ne_k[i]; }
       const int ip = ne & 1;
-      ok = mbar_wait_warp(&item_done[k][ip], (uint32_t)((ne >> 1) & 1), status);
-      ok = ok && mbar_wait_warp(&st_full[k][ip], (uint32_t)((ne >> 1) & 1), status);
+      ok = mbar_wait_then_vote(&item_done[k][ip], (uint32_t)((ne >> 1) & 1), status);
+      ok = ok && mbar_wait_then_vote(&st_full[k][ip], (uint32_t)((ne >> 1) & 1), status);
       if (!ok) break;
       tc_fence_after();
       float ms[GH], ls[GH], ys[GH];
@@ -663,7 +668,7 @@ mala_decode_fp8_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       if (publisher) { xch[k][half][xb][w][pub_row] = mx_w; xch[k][half][xb][w][8 + pub_row] = psum_w; }
       __syncwarp();
       if (lane == 0) mbar_arrive(&grp_bar[k][half]);
-      const bool kk = mbar_wait_warp(&grp_bar[k][half], xc & 1, status);
+      const bool kk = kSplit ? mbar_wait_then_vote(&grp_bar[k][half], xc & 1, status) : mbar_wait_warp(&grp_bar[k][half], xc & 1, status);
       ++xc;
       if (!kk) return false;
       float a0[GS], a1[GS], a2[GS], a3[GS];

@@ -88,6 +88,13 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, i
   }
 }
 
+// The same with one vote at the end: each lane polls by itself, so that a poll is a test alone.  Slower where the phase is complete
+// (see above), better in a warp that mostly waits long beside warps that compute (see its callers).
+__device__ __forceinline__ bool mbar_wait_then_vote(uint64_t* bar, uint32_t parity, int* status) {
+  const bool ok = mbar_wait(bar, parity, status);
+  return __all_sync(0xffffffffu, ok);
+}
+
 // The same for a warp that shares its scheduler with warps doing arithmetic: between two tests it sleeps for a few
 // dozen nanoseconds, so that its polling does not take their issue slots.
 __device__ __forceinline__ bool mbar_wait_warp_idle(uint64_t* bar, uint32_t parity, int* status) {
