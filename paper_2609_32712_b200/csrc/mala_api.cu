@@ -69,11 +69,21 @@ static bool set_smem(K kernel, int bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
 }
 
+// The tiles of mala_fwd_one_kernel begin where its dynamic shared memory does, and have to begin on a 1024-byte boundary: they do as
+// long as the kernel has no static shared memory and the system's part in front is whole kilobytes.
+template <class K>
+static bool set_smem_one_of(K kernel, int bytes) {
+  cudaFuncAttributes a;
+  int dev = 0, reserved = 0;
+  return cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess && reserved % 1024 == 0 &&
+         cudaFuncGetAttributes(&a, kernel) == cudaSuccess && a.sharedSizeBytes == 0 && set_smem(kernel, bytes);
+}
 template <int D>
 static bool set_smem_one() {
   constexpr int bytes = FwdOneCfg<D>::kSmemBytes;
-  return set_smem(mala_fwd_one_kernel<D, true>, bytes) && set_smem(mala_fwd_one_kernel<D, false>, bytes) &&
-         set_smem(mala_fwd_one_kernel<D, true, true>, bytes) && set_smem(mala_fwd_one_kernel<D, false, true>, bytes);
+  return set_smem_one_of(mala_fwd_one_kernel<D, true>, bytes) && set_smem_one_of(mala_fwd_one_kernel<D, false>, bytes) &&
+         set_smem_one_of(mala_fwd_one_kernel<D, true, true>, bytes) && set_smem_one_of(mala_fwd_one_kernel<D, false, true>, bytes);
 }
 
 // SMs of a device, asked for once.
