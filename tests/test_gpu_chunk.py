@@ -306,6 +306,14 @@ def test_chunk_split_skipping_regime(mala, oracle, Nk, Nq, S, tau):
     assert _run_split(mala, oracle, _chunk(w, Nq), tau, S) > 0, "workload must exercise skipping"
 
 
+@pytest.mark.parametrize("tau", [0.0, 1e-3])
+@pytest.mark.parametrize("Nk,Nq,d,Hq,S", [(1500, 476, 128, 12, 4), (1500, 348, 64, 20, 3), (1500, 348, 96, 20, 3)])
+def test_chunk_split_two_query_blocks_per_cta(mala, oracle, Nk, Nq, d, Hq, S, tau):
+    # (more blocks over all heads and ranges than SMs; a ragged last one, with 348 queries the third)
+    w = W.custom_prefill(1, Hq, 4, Nk, d, head_types=["diffuse", "peaked", "peaked", "sink"] * (Hq // 4), seed=Nq, preset="R")
+    _run_split(mala, oracle, _chunk(w, Nq), tau, S)
+
+
 def test_chunk_split_non_causal(mala, oracle):
     w = W.custom_prefill(1, 2, 1, 1100, 128, head_types=["peaked", "diffuse"], seed=5, preset="R")
     _run_split(mala, oracle, _chunk(w, 200), 1e-2, 3, causal=False)

@@ -62,11 +62,35 @@ def test_fwd_small_shapes_literal(mala, oracle, N, d, Hq, Hkv, tau):
 
 
 @pytest.mark.parametrize("tau", [0.0, 1e-3])
-@pytest.mark.parametrize("N,d,H", [(130, 64, 74), (130, 64, 75), (300, 128, 49), (300, 128, 50)])
+@pytest.mark.parametrize("N,d,H", [(130, 64, 74), (130, 64, 75), (300, 128, 49), (300, 128, 50), (130, 64, 148), (130, 64, 149),
+                                   (300, 128, 98), (300, 128, 99), (300, 96, 98), (300, 96, 99)])
 def test_fwd_one_or_two_blocks_per_cta(mala, oracle, N, d, H, tau):
-    # as many query blocks as a GPU of 148 SMs has SMs (a CTA each), and just more of them (two per CTA)
+    # on a GPU of 148 SMs: one query block per SM and just more of them; two per SM (up to here a CTA has one block) and just more
     w = W.custom_prefill(1, H, H, N, d, seed=N + H, preset="R")
     _run_and_check(mala, oracle, w, tau)
+
+
+@pytest.mark.parametrize("tau", [0.0, 1e-3])
+@pytest.mark.parametrize("N,d,H", [(130, 64, 74), (130, 64, 75), (300, 128, 49), (300, 128, 50)])
+def test_fwd_one_or_two_blocks_per_cta_non_causal(mala, oracle, N, d, H, tau):
+    # (here a CTA has one block up to one query block per SM)
+    w = W.custom_prefill(1, H, H, N, d, seed=N + H, preset="R")
+    _run_and_check(mala, oracle, w, tau, causal=False)
+
+
+@pytest.mark.parametrize("tau", [0.0, 1e-5, 1e-3])
+@pytest.mark.parametrize("N,d", [(1000, 128), (1100, 64), (900, 96)])
+def test_fwd_rows_are_the_same_whichever_kernel_takes_them(mala, N, d, tau):
+    # 8 blocks of 4 heads: one block per CTA; the same heads among 80 of them: two per CTA (on any GPU of up to 300 SMs)
+    w = W.custom_prefill(1, 80, 80, N, d, head_types=["diffuse", "sink", "peaked", "planted"] * 20, seed=N, preset="R", device="cuda")
+    q, k, v = (w[x] for x in ("q", "k", "v"))
+    o, lse, st = mala.fwd(q, k, v, w["scale"], tau, stats=True)
+    T = -(-N // 128)
+    for h in (0, 40, 76):
+        o1, lse1, st1 = mala.fwd(*(x[:, :, h:h + 4].contiguous() for x in (q, k, v)), w["scale"], tau, stats=True)
+        assert torch.equal(o1, o[:, :, h:h + 4]) and torch.equal(lse1, lse[:, h:h + 4])
+        assert torch.equal(st1.mask(T), st.mask(T)[:, h:h + 4])
+    assert mala.device_status() == 0
 
 
 @pytest.mark.parametrize("tau", [1e-5, 1e-4, 1e-3, 1.0])

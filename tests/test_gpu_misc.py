@@ -162,6 +162,48 @@ def test_calls_can_be_captured_in_a_cuda_graph(mala):
     assert torch.equal(o_g, o_d) and torch.equal(po_g, po_d) and torch.equal(plse_g, plse_d)
 
 
+@pytest.mark.parametrize("N,d,Hq,Hkv,tau", [(600, 128, 4, 2, 0.0), (600, 64, 2, 2, 1e-4), (2500, 128, 4, 1, 1e-4),
+                                            (12300, 128, 2, 1, 1e-4)])
+def test_backward_captured_and_on_a_side_stream(mala, N, d, Hq, Hkv, tau):
+    """The backward's launches follow one another as programmatic dependents in places: dense; one kernel that tests as it
+    goes; a first pass and the list; and these with the kernel for the rows that retain everything behind them.  Each is
+    captured, replayed on new inputs in the same buffers, and compared with direct calls on another stream."""
+    w = W.custom_prefill(1, Hq, Hkv, N, d, head_types=["diffuse", "peaked"] * (Hq // 2), seed=N, preset="R", device="cuda")
+    q, k, v, do = (w[x] for x in ("q", "k", "v", "do"))
+    o, lse, _ = mala.fwd(q, k, v, w["scale"], tau)
+    dq, dk, dv = (torch.zeros_like(x) for x in (q, k, v))
+    ws = torch.empty(mala.workspace_bytes(mala.OP_BWD, 1, Hq, Hkv, N, d), dtype=torch.uint8, device="cuda")
+
+    def step():
+        mala.fwd(q, k, v, w["scale"], tau, out=o, lse=lse)
+        mala.bwd(q, k, v, o, do, lse, w["scale"], tau, dq=dq, dk=dk, dv=dv, ws=ws)
+
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        step()
+    torch.cuda.current_stream().wait_stream(side)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+        step()                                      # (the second one reuses the scratch of the first)
+    q.copy_(torch.roll(q, 3, dims=1))
+    do.copy_(torch.roll(do, 5, dims=1))
+    graph.replay()
+    torch.cuda.synchronize()
+    got = [x.clone() for x in (dq, dk, dv)]
+    with torch.cuda.stream(side):
+        o2, lse2, _ = mala.fwd(q, k, v, w["scale"], tau)
+        want = mala.bwd(q, k, v, o2, do, lse2, w["scale"], tau)[:3]
+    torch.cuda.synchronize()
+    assert mala.device_status() == 0
+    assert torch.equal(o, o2) and torch.equal(lse, lse2)
+    # dK, dV: the same order of additions, the same bits; dQ: fp32 additions of up to 97 tiles in another order, then one
+    # rounding to bf16 (2^-8 of a value at most where it falls the other way)
+    assert torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+    assert parity.rel_l2(got[0].float().cpu().numpy(), want[0].float().cpu().numpy()) <= 2.0 ** -8
+
+
 def test_autograd_function_runs_both_algorithms(mala, oracle):
     from paper_2609_32712_b200.autograd import mala_attention
     w = W.custom_prefill(1, 4, 2, 640, 128, head_types=["diffuse", "peaked", "peaked", "sink"], seed=41, preset="R")

@@ -93,6 +93,14 @@ def test_varlen_skipping_regime(mala, oracle, tau):
     assert sk > 0, "workload must exercise skipping"
 
 
+@pytest.mark.parametrize("tau", [0.0, 1e-3])
+@pytest.mark.parametrize("d,causal", [(64, True), (96, True), (128, True), (128, False)])
+def test_varlen_with_two_query_blocks_per_cta(mala, oracle, d, causal, tau):
+    # 6 sequences of up to 5 blocks, 12 heads: more blocks than where a CTA is given one (the small calls have that kernel)
+    _run(mala, oracle, [517, 130, 640, 1, 333, 257], 12, 4, d, tau, preset="R", causal=causal,
+         head_types=["diffuse", "peaked", "peaked", "sink"] * 3)
+
+
 @pytest.mark.parametrize("tau", [0.0, 1e-2])
 def test_varlen_non_causal(mala, oracle, tau):
     # every key of the sequence legal: the rows of the next sequence inside a sequence's last tile must be masked
@@ -240,11 +248,20 @@ def test_varlen_prefix_backward_sequences_without_queries_get_zero_gradients(mal
 @pytest.mark.parametrize("page,d", [(128, 128), (256, 128), (16, 128), (64, 128), (8, 64), (32, 96), (128, 40),
                                     (256, 256), (16, 256), (128, 200), (8, 256), (8, 136)])
 def test_prefill_chunks_against_a_paged_cache(mala, oracle, tau, page, d):
+    _run_paged(mala, oracle, tau, page, d, 4, 2)
+
+
+@pytest.mark.parametrize("tau", [0.0, 1e-4])
+@pytest.mark.parametrize("page,d", [(128, 128), (16, 128), (64, 64), (16, 96), (128, 64)])
+def test_prefill_chunks_against_a_paged_cache_two_query_blocks_per_cta(mala, oracle, tau, page, d):
+    _run_paged(mala, oracle, tau, page, d, 16, 4)          # (4 sequences of up to 3 blocks: 192, more than SMs)
+
+
+def _run_paged(mala, oracle, tau, page, d, Hq, Hkv):
     """Packed prefill chunks whose keys and values (prefix and chunk) lie in pages scattered over a shuffled pool."""
-    Hq, Hkv = 4, 2
     nk = [900, 128, 517, 300]
     nq = [260, 128, 100, 1]
-    ws = [W.custom_prefill(1, Hq, Hkv, n, d, head_types=["diffuse", "peaked", "peaked", "sink"], seed=70 + x, preset="R")
+    ws = [W.custom_prefill(1, Hq, Hkv, n, d, head_types=["diffuse", "peaked", "peaked", "sink"] * (Hq // 4), seed=70 + x, preset="R")
           for x, n in enumerate(nk)]
     Nmax = -(-max(nk) // page) * page
     kc = torch.zeros((len(nk), Nmax, Hkv, d), dtype=torch.bfloat16)
