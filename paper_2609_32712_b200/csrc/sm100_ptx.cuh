@@ -162,7 +162,8 @@ inline int order_by_size(long long bytes, long long most, long long blocks, int 
 __device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launches `kernel`, which begins with wait_for_primary(), as a programmatic dependent of the kernel before it.  A launch that
+// Launches `kernel` as a programmatic dependent of the kernel before it: it calls wait_for_primary() before it touches what that
+// one writes or reads, and every block of it does so before it ends, so that it is never over before that one is.  A launch that
 // fails is reported here alone: the runtime's last error is taken back, so that the next call's check does not meet it.
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
