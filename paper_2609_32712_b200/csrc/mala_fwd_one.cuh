@@ -14,7 +14,7 @@
 //
 // 16 / 4 heads of 256 columns, 8192 tokens, every tile retained: 426 us dense and 456 with the test; 727 and 757 with one score
 // buffer, one thread per row and a stage of a whole tile each for K and V (a quarter of the tiles retained: 334, 519).  There the
-// tensor pipe is 86 % busy until the power limit sets in; with 64 and 128 columns the chain of 2100-2800 clk per tile is the bound.
+// MMAs take 2048 of the 2390 clk per tile until the power limit sets in; with 64 and 128 columns the chain of 2100-2800 clk per tile is the bound.
 //
 // Warp roles (384 threads): warp 0 K copies (and Q), warp 1 UMMA issuer, warp 2 V copies, warp 3 idle, warps 4-7 / 8-11 the
 // softmax threads of the tile's first / second 64 keys.  All synchronisation is by mbarriers and polls with bounded waits.
